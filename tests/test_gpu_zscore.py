@@ -80,3 +80,54 @@ def test_deterministic_and_rejects_bad_arguments():
         with pytest.raises(B.MLPError) as e:
             B.mlp_zscore(dev(X[:10]), 10, 33, n_fit, B.MLP_FP32, D_out, Y, m, m, W, wsb, stream())
         assert e.value.status == B.MLP_EINVAL
+
+
+@pytest.mark.parametrize("n,D", [(200_003, 33), (120_001, 5), (60_000, 17), (90_001, 300)])
+def test_statistics_of_long_tables_and_extreme_columns(n, D):
+    """Row counts where a block's rows are added in groups of 16 and 4 with a
+    remainder, with columns outside the range of the groups' FP32 sums: huge,
+    tiny, constant, offset by 1e7 deviations, infinite and NaN.  Finite columns
+    against numpy's 64-bit sums: an FP64 sum of n terms in blocks of a few
+    hundred rows is within 1e-12 of it; the mean of a column centred on 0 is
+    that much of its deviation, and the deviation of the offset column carries
+    the 1e7 of its offset in the mean's rounding only (1e-12 holds)."""
+    X = table(11 + D, n, D).astype(np.float64)
+    rng = np.random.default_rng(5)
+    X[:, 0] = rng.normal(size=n) * 1e30
+    X[:, 1] = rng.normal(size=n) * 1e-30
+    X[:, 2] = np.float32(1e4) + rng.normal(size=n) * 1e-3
+    X[5, D - 1] = np.inf if D > 5 else 1.0
+    if D > 5:
+        X[n // 2, D - 2] = np.nan
+    X = X.astype(np.float32)
+    Y, m, s = run(X, n, B.MLP_FP32, D)
+    X = X.astype(np.float64)
+    ok = np.isfinite(X).all(0)
+    mr, sr = X.mean(0), X.std(0)
+    assert np.all(np.abs(m - mr)[ok] <= 1e-12 * (np.abs(mr) + sr)[ok])
+    np.testing.assert_allclose(s[ok], sr[ok], rtol=1e-12, atol=0)
+    assert s[3] == 0.0 and np.all(Y[:, 3] == 0.0)
+    if D > 5:
+        assert np.isposinf(m[D - 1]) and np.isnan(m[D - 2]) and np.isnan(s[D - 1]) and np.isnan(s[D - 2])
+
+
+@pytest.mark.parametrize("prec,D,D_out,n", [(B.MLP_FP32, 33, 33, 64), (B.MLP_FP32, 33, 35, 129), (B.MLP_FP32, 3, 3, 7),
+                                            (B.MLP_BF16, 33, 37, 65), (B.MLP_BF16, 256, 256, 19), (B.MLP_FP32, 5, 21, 1000),
+                                            (B.MLP_BF16, 257, 264, 9), (B.MLP_FP32, 1, 300, 300)])
+def test_tiled_and_plain_apply_agree(prec, D, D_out, n):
+    """16-byte aligned buffers (tiles) and buffers one element off (an element
+    a thread): the same bits for every width, remainder and padding."""
+    import torch
+    X = dev(table(17 + n, n, D))
+    ws = B.mlp_zscore_workspace_bytes(D)
+    W = torch.empty(ws, dtype=torch.uint8, device="cuda")
+    m = torch.zeros(D, dtype=torch.float64, device="cuda")
+    s = torch.zeros(D, dtype=torch.float64, device="cuda")
+    dt = torch.int32 if prec == B.MLP_FP32 else torch.int16
+    out = []
+    for off in (0, 1):
+        buf = torch.full((n * D_out + 2,), 99, dtype=dt, device="cuda")
+        B.mlp_zscore(X, n, D, n, prec, D_out, buf[off:off + n * D_out], m, s, W, ws, stream())
+        out.append(host(buf[off:off + n * D_out]))
+        assert int(buf[off + n * D_out]) == 99
+    assert np.array_equal(out[0], out[1])
