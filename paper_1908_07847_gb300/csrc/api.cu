@@ -142,9 +142,9 @@ mlp_status ensure_plain(mlp_t h, int64_t n, bool need_hid, mlp::PlainWork *w) {
 double loss_scale(int loss_mean, int64_t n) { return loss_mean ? (n > 0 ? 1.0 / (double)n : 0.0) : 1.0; }
 
 // One plain-path gradient evaluation into the handle's packed gradient buffer
-// (or caller pointers); loss (may be NULL) = 0.5 * c_loss * sse.
+// (or caller pointers); fin says what else becomes of it and of the loss.
 mlp_status plain_grad(mlp_t h, const void *X, const void *y, int64_t n, void *gW1, void *gb1, void *gw2,
-                      void *gb2, double *loss, double c_loss, cudaStream_t st) {
+                      void *gb2, const mlp::PlainFinish &fin, cudaStream_t st) {
     mlp::PlainWork w;
     mlp_status s = ensure_plain(h, n, true, &w);
     if (s) return s;
@@ -153,9 +153,29 @@ mlp_status plain_grad(mlp_t h, const void *X, const void *y, int64_t n, void *gW
                           h->hid, h->obuf, y, nullptr, c, w, st),
        "forward kernels");
     CK(mlp::plain_backward(h->cfg.prec, h->cfg.act, h->cfg.D, h->cfg.H, n, X, W1p(h), w2p(h), h->hid, gW1, gb1,
-                           gw2, gb2, nullptr, loss, c_loss, h->status, w, st),
+                           gw2, gb2, nullptr, fin, w, st),
        "backward kernels");
     return MLP_OK;
+}
+
+// Loss c_loss / 2 x sse into *loss (may be NULL), the handle's own status word.
+mlp::PlainFinish finish_loss(mlp_t h, double *loss, double c_loss) {
+    mlp::PlainFinish f;
+    f.loss = loss;
+    f.c_loss = c_loss;
+    f.status = h->status;
+    return f;
+}
+
+// The same with the update of the handle's weights.
+mlp::PlainFinish finish_step(mlp_t h, double *loss, double c_loss) {
+    mlp::PlainFinish f = finish_loss(h, loss, c_loss);
+    f.W1 = W1p(h);
+    f.b1 = b1p(h);
+    f.w2 = w2p(h);
+    f.b2 = b2p(h);
+    f.lr = (double)h->cfg.lr;
+    return f;
 }
 
 mlp_status check_handle(mlp_t h) {
@@ -292,7 +312,7 @@ mlp_status mlp_backward(mlp_t h, const void *X, const void *y, int64_t n, void *
     if (n < 0 || !gW1 || !gb1 || !gw2 || !gb2 || (n > 0 && (!X || !y)))
         return fail(MLP_EINVAL, "mlp_backward: bad arguments");
     DeviceScope ds(h->device);
-    return plain_grad(h, X, y, n, gW1, gb1, gw2, gb2, loss, loss_scale(h->cfg.loss_mean, n),
+    return plain_grad(h, X, y, n, gW1, gb1, gw2, gb2, finish_loss(h, loss, loss_scale(h->cfg.loss_mean, n)),
                       (cudaStream_t)stream);
 }
 
@@ -312,13 +332,8 @@ mlp_status mlp_step_plain(mlp_t h, const void *X, const void *y, int64_t n, doub
     if (n < 0 || (n > 0 && (!X || !y))) return fail(MLP_EINVAL, "mlp_step_plain: bad arguments");
     DeviceScope ds(h->device);
     cudaStream_t st = (cudaStream_t)stream;
-    mlp_status s = plain_grad(h, X, y, n, gW1p(h), gb1p(h), gw2p(h), gb2p(h), loss,
-                              loss_scale(h->cfg.loss_mean, n), st);
-    if (s) return s;
-    CK(mlp::plain_update(h->cfg.prec, h->cfg.D, h->cfg.H, (double)h->cfg.lr, W1p(h), b1p(h), w2p(h), b2p(h),
-                         gW1p(h), gb1p(h), gw2p(h), gb2p(h), st),
-       "mlp_step_plain update");
-    return MLP_OK;
+    return plain_grad(h, X, y, n, gW1p(h), gb1p(h), gw2p(h), gb2p(h),
+                      finish_step(h, loss, loss_scale(h->cfg.loss_mean, n)), st);
 }
 
 mlp_status mlp_train_epochs(mlp_t h, const void *X, const void *y, int64_t n, int32_t epochs, int64_t minibatch,
@@ -381,19 +396,15 @@ mlp_status mlp_train_epochs(mlp_t h, const void *X, const void *y, int64_t n, in
     const double C = loss_scale(h->cfg.loss_mean, n);
     const size_t xb = x_elem_bytes(h->cfg.prec) * (size_t)D;
     for (int e = 0; e < epochs; ++e) {
-        int first = 1;
         for (int64_t b0 = 0; b0 < n; b0 += mbs) {
             const int64_t m = (n - b0) < mbs ? (n - b0) : mbs;
+            mlp::PlainFinish f = finish_step(h, loss_hist ? loss_hist + e : h->dtmp + 64, C);
+            f.loss_add = loss_hist && b0 > 0;
             mlp_status s = plain_grad(h, (const char *)X + xb * b0, (const char *)y + h->esz * b0, m, gW1p(h),
-                                      gb1p(h), gw2p(h), gb2p(h), h->dtmp + 64, C, st);
+                                      gb1p(h), gw2p(h), gb2p(h), f, st);
             if (s) return s;
             if (gnorm_hist && b0 + mbs >= n)
                 CK(mlp::plain_gnorm(h->cfg.prec, h->P, h->grads, h->dtmp, gnorm_hist + e, st), "gnorm");
-            CK(mlp::plain_update(h->cfg.prec, D, H, (double)h->cfg.lr, W1p(h), b1p(h), w2p(h), b2p(h), gW1p(h),
-                                 gb1p(h), gw2p(h), gb2p(h), st),
-               "update");
-            if (loss_hist) CK(mlp::plain_accum(loss_hist + e, h->dtmp + 64, first, st), "loss");
-            first = 0;
         }
     }
     return MLP_OK;
@@ -563,8 +574,7 @@ mlp_status mlp_backward_w(int32_t prec, int32_t act, int32_t D, int32_t H, int64
     mlp::plain_workspace_carve(workspace, prec, D, H, n, mlp::device_sm_count(), &w);
     cudaStream_t st = (cudaStream_t)stream;
     if (n > 0) CK(mlp::plain_d2_upstream(prec, n, o, dLdo, w.d2, st), "mlp_backward_w d2");
-    CK(mlp::plain_backward(prec, act, D, H, n, X, W1, w2, hid, gW1, gb1, gw2, gb2, gX, nullptr, 0.0, nullptr, w,
-                           st),
+    CK(mlp::plain_backward(prec, act, D, H, n, X, W1, w2, hid, gW1, gb1, gw2, gb2, gX, mlp::PlainFinish(), w, st),
        "mlp_backward_w");
     return MLP_OK;
 }

@@ -175,14 +175,22 @@ cudaError_t plain_forward(int prec, int act, int D, int H, int64_t n, const void
                           void *hid, void *o, const void *y, const void *dLdo, double c,
                           const PlainWork &w, cudaStream_t st);
 
+// What becomes of the gradient besides the four arrays it is written to.
+struct PlainFinish {
+    void *W1 = nullptr, *b1 = nullptr, *w2 = nullptr, *b2 = nullptr;  // if given: w -= lr g
+    double lr = 0.0;
+    double *loss = nullptr;      // if given: 0.5 c_loss sse is stored, or
+    bool loss_add = false;       //   added, there
+    double c_loss = 0.0;
+    int *status = nullptr;       // if given: ST_NONFINITE for a loss that is not finite
+};
+
 // Gradient partials and their fixed-order reduction into gW1, gb1, gw2, gb2.
-// Needs hid and d2 from plain_forward.  loss (may be NULL) = 0.5 c_loss sse.
-// gX (may be NULL) = d1 W1.
+// Needs hid and d2 from plain_forward.  gX (may be NULL) = d1 W1.
 cudaError_t plain_backward(int prec, int act, int D, int H, int64_t n, const void *X,
                            const void *W1, const void *w2, const void *hid,
                            void *gW1, void *gb1, void *gw2, void *gb2, void *gX,
-                           double *loss, double c_loss, int *status,
-                           const PlainWork &w, cudaStream_t st);
+                           const PlainFinish &fin, const PlainWork &w, cudaStream_t st);
 
 // w <- w - lr g over the four parameter arrays.
 cudaError_t plain_update(int prec, int D, int H, double lr, void *W1, void *b1, void *w2,
@@ -195,9 +203,6 @@ cudaError_t plain_gnorm(int prec, int64_t P, const void *g_packed, double *scrat
 
 // d2 = dLdo o (1 - o) into w.d2 (autograd backward).
 cudaError_t plain_d2_upstream(int prec, int64_t n, const void *o, const void *dLdo, void *d2, cudaStream_t st);
-
-// *dst = (first ? 0 : *dst) + *src (one thread).
-cudaError_t plain_accum(double *dst, const double *src, int first, cudaStream_t st);
 
 // labels[i] = o_i >= 0.5
 cudaError_t plain_labels(int prec, int64_t n, const void *o, int8_t *labels, cudaStream_t st);

@@ -1,0 +1,64 @@
+"""The general kernels (any D and H) at the edges of their tiles: row tiles of
+16 to 128 rows picked by the grid's size, inputs staged in slices of up to 64,
+gradient tiles of 64 inputs in quads with 2 to 32 row subsets, input-gradient
+row groups; forward, upstream-gradient backward and a training step against the
+oracle at the FP32 bars (1e-12 in FP64)."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import Params
+from paper_1908_07847_gb300 import binding as B
+from tests.gpu_util import FWD_TOL, GRAD_TOL, W_TOL, Net, dev, host, lr32, problem, rel_err_elem, rel_err_norm, stream
+
+pytestmark = pytest.mark.gpu
+
+#        rows, D, H: one row; slices 65 = 33 + 32; 128-row tiles; 64-row tiles; two
+#        input tiles; three; one quad; quads of 2 inputs with 16 subsets; aligned hid
+SHAPES = [(1, 1, 1), (33, 65, 65), (40001, 36, 70), (20003, 33, 64), (2500, 65, 300), (77, 130, 67), (513, 3, 129),
+          (1025, 7, 31), (4096, 64, 512), (17, 64, 130), (15, 49, 200)]
+
+
+@pytest.mark.parametrize("n,D,H", SHAPES)
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+def test_forward_and_upstream_gradients(n, D, H, dtype):
+    import torch
+    from paper_1908_07847_gb300.autograd import mlp
+    if dtype == "float64" and n * D * H > 4e7:
+        n = 3001
+    act = (n + H) % 2
+    X, _, W = problem(7000 + n + H, n, D, H)
+    dt = getattr(torch, dtype)
+    rng = np.random.default_rng(n)
+    go = rng.normal(size=n).astype(np.float32)
+    t = [dev(np.asarray(a, np.float32)).to(dt).requires_grad_(True) for a in (X, *W)]
+    o = mlp(*t, act)
+    g = torch.autograd.grad(o, t, dev(go).to(dt))
+    p = Params(*[np.asarray(a, np.float64) for a in W])
+    _, o_ref = oracle.forward(X, p, act)
+    gW1, gb1, gw2, gb2, gX = oracle.backward(X, p, go.astype(np.float64), act, want_gX=True)
+    ft, gt = (FWD_TOL, GRAD_TOL) if dtype == "float32" else (1e-12, 1e-12)
+    assert rel_err_elem(host(o), o_ref) <= ft
+    for got, want in zip(g, (gX, gW1, gb1, gw2, gb2)):
+        assert rel_err_norm(host(got), want) <= gt
+
+
+@pytest.mark.parametrize("n,D,H,mb", [(300, 70, 129, 0), (1000, 33, 300, 260), (65, 64, 513, 64)])
+@pytest.mark.parametrize("loss_mean", [0, 1])
+def test_training_steps_update_and_loss(n, D, H, mb, loss_mean):
+    """Gradient reduction, update and loss in one kernel: weights, loss and
+    gradient-norm histories of three epochs against the oracle."""
+    import torch
+    X, y, W = problem(7100 + n, n, D, H)
+    lr = 0.1 if loss_mean else 0.1 / n
+    lh = torch.zeros(3, dtype=torch.float64, device="cuda")
+    gh = torch.zeros(3, dtype=torch.float64, device="cuda")
+    with Net(D, H, lr=lr, loss_mean=loss_mean) as net:
+        net.set(W)
+        B.mlp_train_epochs(net.h, dev(X), dev(y), n, 3, mb, lh, gh, stream())
+        assert net.check() == B.MLP_OK
+        got = net.flat()
+    q, l_ref, g_ref = oracle.train(X, y, Params(*W), lr32(lr), 3, minibatch=mb, loss_mean=bool(loss_mean))
+    assert rel_err_norm(got, q.flat()) <= W_TOL
+    np.testing.assert_allclose(host(lh), l_ref, rtol=1e-6)
+    np.testing.assert_allclose(host(gh), g_ref, rtol=1e-4)
