@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <algorithm>
@@ -36,7 +37,7 @@ struct mlp_net {
     double *gnp = nullptr;    // per-epoch gradient-norm partials (tensor-core cluster path)
     size_t gnp_cap = 0;
     int skip_block = -1;
-    int rows_per_block = 32;
+    int rows_per_block = 0;   // fused kernel: 0 = by the step's size
     int max_clusters = 1 << 30;   // cap on clusters of the tensor-core kernel
     mlp::FusedCounters ctr;   // fused-kernel counter values at the next launch
 };
@@ -192,10 +193,16 @@ namespace mlp {
 mlp_status set_error(mlp_status s, const char *msg) { return fail(s, "%s", msg); }
 
 int device_sm_count() {
+    // per device, asked once (a property of the hardware; every launch asks)
+    constexpr int MAXDEV = 64;
+    static std::atomic<int> cache[MAXDEV];
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (dev >= 0 && dev < MAXDEV && (n = cache[dev].load(std::memory_order_relaxed)) > 0) return n;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-    return n > 0 ? n : 1;
+    if (n < 1) n = 1;
+    if (dev >= 0 && dev < MAXDEV) cache[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 }  // namespace mlp
 

@@ -16,13 +16,14 @@ namespace {
 constexpr int BNT = RE_NT;       // threads per block
 constexpr int BCAP = 256;        // rows staged in shared memory at a time
 
-template <int DP, int WU, int ACT>
+constexpr int RING = 32;         // epochs whose losses are finished together
+
+// RB1, RBN: rows a lane keeps in flight for H <= 32 and above.
+template <int DP, int WU, int ACT, int RB1, int RBN, bool ONE>
 __device__ __forceinline__ void net_body(const BatchNet &nd, int D, int epochs, float lr, int loss_mean,
                                          int *status, float *Xs, float *ys, float *Wm, float *part,
-                                         float *zx, double *s_sse, double *s_gn) {
-    // One row in flight per lane for H <= 32: at two blocks per SM the second
-    // row's registers spill (measured 4.7 % slower on the 4096-net workload).
-    using Eng = RowEngine<DP, WU, ACT, 1>;
+                                         float *zx, double (*s_sse)[RE_NW], double *s_gn) {
+    using Eng = RowEngine<DP, WU, ACT, RB1, RBN>;
     Eng eng;
     eng.setup(nd.H, D);
     constexpr int NG = Eng::NG;
@@ -45,6 +46,21 @@ __device__ __forceinline__ void net_body(const BatchNet &nd, int D, int epochs, 
     const float c = loss_mean ? 1.0f / (float)n : 1.0f;
     const double C = loss_mean ? 1.0 / (double)n : 1.0;
 
+    // The loss of epochs first.. (warp 0): a dozen dependent FP64 operations each.
+    // ONE: RING epochs' at a time, a lane each, while the next epoch runs; with
+    // two blocks an SM the other block fills that gap, and the registers this
+    // takes cost more (2 to 6 %).
+    constexpr int HELD = ONE ? RING : 1;
+    auto finish_losses = [&](int first, int cnt) {
+        if (tid < cnt) {
+            const double *v = s_sse[(first + tid) & (2 * HELD - 1)];
+            double t = 0.0;
+            for (int q = 0; q < NG; ++q) t += v[q];
+            const double L = 0.5 * C * t;
+            if (nd.loss_hist) nd.loss_hist[first + tid] = L;
+            if (!isfinite(L)) atomicOr(status, ST_NONFINITE);
+        }
+    };
     for (int e = 0; e < epochs; ++e) {
         eng.load_weights(Wm);
         for (int64_t cs = 0; cs < n; cs += BCAP) {
@@ -56,7 +72,7 @@ __device__ __forceinline__ void net_body(const BatchNet &nd, int D, int epochs, 
             }
             eng.rows(Xs, ys, cn, c, zx);
         }
-        eng.write_group(part, s_sse);
+        eng.write_group(part, s_sse[e & (2 * HELD - 1)]);
         __syncthreads();
         // Update, and the FP64 squared norm of the gradient it applies: each
         // thread's values in index order, then a fixed butterfly per warp and
@@ -64,43 +80,54 @@ __device__ __forceinline__ void net_body(const BatchNet &nd, int D, int epochs, 
         // (FP64 arithmetic is slow on this part: only when asked for.)
         double gn = 0.0;
         const bool want_gn = nd.gnorm_hist != nullptr;
-        for (int p = tid; p < P; p += BNT) {
-            float g = part[p];
+        constexpr int PF = ONE ? 4 : 1;   // parameters in flight a thread
+        for (int base = tid; base < P; base += PF * BNT) {
+            float g[PF];
 #pragma unroll
-            for (int q = 1; q < NG; ++q) g += part[q * P + p];
-            Wm[p] -= lr * g;
-            if (want_gn) gn = fma((double)g, (double)g, gn);
+            for (int u = 0; u < PF; ++u) {
+                const int p = PF > 1 ? min(base + u * BNT, P - 1) : base;
+                g[u] = part[p];
+#pragma unroll
+                for (int q = 1; q < NG; ++q) g[u] += part[q * P + p];
+            }
+#pragma unroll
+            for (int u = 0; u < PF; ++u) {
+                const int p = base + u * BNT;
+                if (PF > 1 && p >= P) break;
+                Wm[p] -= lr * g[u];
+                if (want_gn) gn = fma((double)g[u], (double)g[u], gn);
+            }
         }
         if (want_gn) {
             gn = warp_sum(gn);
             if ((tid & 31) == 0) s_gn[tid >> 5] = gn;
-            __syncthreads();
-        }
-        if (tid == 0) {
-            double t = 0.0;
-            for (int q = 0; q < NG; ++q) t += s_sse[q];
-            const double L = 0.5 * C * t;
-            if (nd.loss_hist) nd.loss_hist[e] = L;
-            if (!isfinite(L)) atomicOr(status, ST_NONFINITE);
-            if (nd.gnorm_hist) {
-                double u = 0.0;
-                for (int q = 0; q < RE_NW; ++q) u += s_gn[q];
-                nd.gnorm_hist[e] = sqrt(u);
-            }
         }
         __syncthreads();
+        if (want_gn && tid == 0) {
+            double u = 0.0;
+            for (int q = 0; q < RE_NW; ++q) u += s_gn[q];
+            nd.gnorm_hist[e] = sqrt(u);
+        }
+        if ((e & (HELD - 1)) == HELD - 1) finish_losses(e + 1 - HELD, HELD);
     }
+    finish_losses(epochs & ~(HELD - 1), epochs & (HELD - 1));
     for (int i = tid; i < P; i += BNT) nd.params[i] = Wm[i];
     __syncthreads();
 }
 
-template <int DP, int ACT>
-__global__ void __launch_bounds__(BNT, (DP <= 36 ? 2 : 1)) k_batched_train(const BatchNet *__restrict__ nets,
+// ONE: one block an SM, for plans of at most one net an SM: a lane then keeps
+// as many rows in flight as the fused kernel's (two subsets of 46 and 44 rows, 16
+// units: 2.92 -> 2.32 us an epoch with the losses finished in groups).  Otherwise two blocks an SM and,
+// for H <= 32, one row in flight: the second row's registers spill there
+// (measured 4.7 % slower on the 4096-net workload).
+template <int DP, int ACT, bool ONE>
+__global__ void __launch_bounds__(BNT, (DP <= 36 && !ONE ? 2 : 1)) k_batched_train(const BatchNet *__restrict__ nets,
                                                          const int *__restrict__ order, int n_nets, int D,
                                                          int epochs, float lr, int loss_mean, int *status,
                                                          int part_floats, int wm_floats) {
+    constexpr int RB1 = ONE && DP <= 36 ? 3 : 1, RBN = ONE ? 8 : RE_RB;
     extern __shared__ __align__(16) float smem[];
-    __shared__ double s_sse[RE_NW];
+    __shared__ double s_sse[2 * RING][RE_NW];
     __shared__ double s_gn[RE_NW];
     float *Xs = smem;                      // BCAP x DP
     float *ys = Xs + BCAP * DP;            // BCAP
@@ -120,18 +147,19 @@ __global__ void __launch_bounds__(BNT, (DP <= 36 ? 2 : 1)) k_batched_train(const
             continue;
         }
         if (nd.H <= 32)
-            net_body<DP, 1, ACT>(nd, D, epochs, lr, loss_mean, status, Xs, ys, Wm, part, zx, s_sse, s_gn);
+            net_body<DP, 1, ACT, RB1, RBN, ONE>(nd, D, epochs, lr, loss_mean, status, Xs, ys, Wm, part, zx, s_sse, s_gn);
         else if (nd.H <= 64)
-            net_body<DP, 2, ACT>(nd, D, epochs, lr, loss_mean, status, Xs, ys, Wm, part, zx, s_sse, s_gn);
+            net_body<DP, 2, ACT, RB1, RBN, ONE>(nd, D, epochs, lr, loss_mean, status, Xs, ys, Wm, part, zx, s_sse, s_gn);
         else
-            net_body<DP, 4, ACT>(nd, D, epochs, lr, loss_mean, status, Xs, ys, Wm, part, zx, s_sse, s_gn);
+            net_body<DP, 4, ACT, RB1, RBN, ONE>(nd, D, epochs, lr, loss_mean, status, Xs, ys, Wm, part, zx, s_sse, s_gn);
     }
 }
 
 template <int DP>
-void *pick(int act) {
-    if (act == MLP_ACT_TANH) return (void *)k_batched_train<DP, MLP_ACT_TANH>;
-    return (void *)k_batched_train<DP, MLP_ACT_SIGMOID>;
+void *pick(int act, bool one) {
+    if (act == MLP_ACT_TANH)
+        return one ? (void *)k_batched_train<DP, MLP_ACT_TANH, true> : (void *)k_batched_train<DP, MLP_ACT_TANH, false>;
+    return one ? (void *)k_batched_train<DP, MLP_ACT_SIGMOID, true> : (void *)k_batched_train<DP, MLP_ACT_SIGMOID, false>;
 }
 
 int dp_for(int D) {
@@ -179,12 +207,13 @@ cudaError_t batched_train(int act, int D, int Hmax, int64_t nmax, const BatchNet
     if (DP == 0 || Hmax > 128) return cudaErrorInvalidValue;
     if (n_nets == 0 || epochs == 0) return cudaSuccess;
     void *fn = nullptr;
+    const bool one = n_nets <= device_sm_count();
     switch (DP) {
-        case 8: fn = pick<8>(act); break;
-        case 16: fn = pick<16>(act); break;
-        case 36: fn = pick<36>(act); break;
-        case 48: fn = pick<48>(act); break;
-        default: fn = pick<64>(act); break;
+        case 8: fn = pick<8>(act, one); break;
+        case 16: fn = pick<16>(act, one); break;
+        case 36: fn = pick<36>(act, one); break;
+        case 48: fn = pick<48>(act, one); break;
+        default: fn = pick<64>(act, one); break;
     }
     int pf, wm;
     size_t smem;

@@ -35,6 +35,7 @@ constexpr int FNT = RE_NT;       // threads per block
 constexpr int CAP = 64;          // rows staged in shared memory at a time
 constexpr int RESIDENT = 192;    // rows a block keeps resident across steps
 constexpr int GMAX = 320;        // largest grid
+constexpr int RING = 32;         // steps of a one-block launch whose losses are finished together
 
 struct FArgs {
     int D, H;
@@ -74,7 +75,8 @@ __device__ __forceinline__ void red_add(long long *p, long long v) {
 
 // One block per SM (the fused grid rarely needs more than one wave): with the
 // register file to itself a lane keeps eight rows in flight for H > 32, and
-// three for H <= 32 with D <= 36, without spilling.
+// three for H <= 32 with D <= 36, without spilling (six, so that 96 rows of a
+// 16-unit net take one turn instead of two, spill 2.4 KB a thread).
 template <int DP, int WU>
 __host__ __device__ constexpr int fused_rb1() { return (WU == 1 && DP <= 36) ? 3 : 2; }
 
@@ -82,6 +84,18 @@ template <int DP, int WU, int ACT>
 __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     extern __shared__ __align__(16) float smem[];
     __shared__ double s_red[RE_NW];
+    // one block: the squared errors of the last steps, by row group, finished
+    // RING steps at a time (two halves: one is finished while the other fills)
+    __shared__ double s_ring[2 * RING][RE_NW];
+    __shared__ double s_val[RING];
+    // kept here rather than in every thread's registers (the row engine fills them)
+    __shared__ struct {
+        int64_t lo[2], hi[2];   // this block's rows of a full step [0] and of the last, ragged one [1]
+        double sse;             // one block: squared error of the epoch so far
+        long long fix;          // several: the same as the sum of the steps' fixed-point values
+        int64_t step;           // one block: of the epoch, the next step to finish
+        int epoch;              //   and its epoch
+    } sv;
     __shared__ long long s_sse;   // the step's fixed-point squared-error sum
     __shared__ double s_gn[RE_NW];
     using Eng = RowEngine<DP, WU, ACT, fused_rb1<DP, WU>(), 8>;
@@ -100,7 +114,23 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     // Rows of a step per block, and whether they stay resident for the launch.
     const int64_t rows_max = cdiv(mbs, G);
     const bool resident = (mbs == a.n) && rows_max <= RESIDENT;
-    const int xcap = resident ? RESIDENT : CAP;
+    // mini-batches whose rows fit CAP: two buffers, the next step's rows load
+    // during this step's reduction, barrier and update
+    const bool ahead = !resident && rows_max <= CAP;
+    const int xcap = resident ? RESIDENT : 2 * CAP;
+    const int64_t nsteps = cdiv(a.n, mbs);
+    if (tid == 0) {   // once: a 64-bit division costs hundreds of cycles
+        const int64_t ml = a.n - (nsteps - 1) * mbs;
+        sv.lo[0] = (mbs * g) / G;
+        sv.hi[0] = (mbs * (g + 1)) / G;
+        sv.lo[1] = (ml * g) / G;
+        sv.hi[1] = (ml * (g + 1)) / G;
+        sv.sse = 0.0;
+        sv.fix = 0;
+        sv.step = 0;
+        sv.epoch = 0;
+    }
+    __syncthreads();
     float *Wm = smem;                               // packed weights
     float *gpart = Wm + wm_floats(D, H);            // NG x P row-group partials
     float *Xs = gpart + re_part_floats(D, H);       // xcap x DP rows
@@ -113,7 +143,6 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     eng.setup(H, D);
     const float gscale = __int_as_float((127 - a.gshift) << 23);   // 2^-gshift
     const float gup = __int_as_float((127 + a.gshift) << 23);      // 2^gshift
-    const double Cl = a.loss_mean ? (a.n > 0 ? 1.0 / (double)a.n : 0.0) : 1.0;
 
     {
         // Initial weights: 16-byte copies through L2, then the tail.
@@ -121,17 +150,17 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
         for (int i = 4 * tid; i < P4; i += 4 * FNT) cp_async16_cg(Wm + i, a.params + i);
         if (tid < P - P4) Wm[P4 + tid] = __ldcg(a.params + P4 + tid);
     }
-    auto stage = [&](int64_t r0, int cn) {
+    auto stage = [&](int64_t r0, int cn, int at) {   // rows r0.. to row `at` of the buffer
         const float *Xg = X + r0 * D;
         for (int i = tid; i < cn * D; i += FNT) {
             const int s = i / D, k = i - s * D;
-            cp_async4(Xs + s * DP + k, Xg + i);
+            cp_async4(Xs + (at + s) * DP + k, Xg + i);
         }
-        for (int i = tid; i < cn; i += FNT) cp_async4(ys + i, Y + r0 + i);
+        for (int i = tid; i < cn; i += FNT) cp_async4(ys + at + i, Y + r0 + i);
     };
-    if (resident) {
-        const int64_t r0 = (mbs * g) / G, r1 = (mbs * (g + 1)) / G;
-        if (r1 > r0) stage(r0, (int)(r1 - r0));
+    if (resident || ahead) {   // the first step's rows
+        const int64_t l = sv.lo[nsteps == 1], h = sv.hi[nsteps == 1];
+        if (h > l) stage(l, (int)(h - l), 0);
     }
     // Only the padding columns D..DP-1 of the row buffer are read without
     // being copied; zero them while the copies are in flight (disjoint words).
@@ -140,27 +169,75 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     cp_async_wait_all();
     __syncthreads();
 
-    double sse_epoch = 0.0;
-    int64_t step = 0;
+    int rot = a.rot;              // accumulator of this step
+    int at = 0;                   // where this step's rows are, when they were loaded ahead
+    int ring = 0;                 // one block: steps done, modulo 2 RING
+    // Finishes `cnt` steps' losses from ring slot `from` (warp 0): as the
+    // cross-block path does, each step's squared error is rounded to 2^-32.
+    auto finish_steps = [&](int from, int cnt) {
+        const double Cl = a.loss_mean ? 1.0 / (double)a.n : 1.0;
+        if (tid < cnt) {
+            double t = 0.0;
+            for (int q = 0; q < NG; ++q) t += s_ring[from + tid][q];
+            const double v = t * 4294967296.0;
+            if (!(v < 4.0e18)) atomicOr(a.status, ST_NONFINITE);
+            s_val[tid] = (double)__double2ll_rn(v) * (1.0 / 4294967296.0);
+        }
+        __syncwarp();
+        if (nsteps == 1) {
+            if (tid < cnt) {
+                const double L = 0.5 * s_val[tid] * Cl;
+                if (a.loss_hist) a.loss_hist[sv.epoch + tid] = L;
+                if (!isfinite(L)) atomicOr(a.status, ST_NONFINITE);
+            }
+            __syncwarp();
+            if (tid == 0) sv.epoch += cnt;
+        } else if (tid == 0) {
+            for (int i = 0; i < cnt; ++i) {
+                sv.sse += s_val[i];
+                if (++sv.step == nsteps) {
+                    const double L = 0.5 * sv.sse * Cl;
+                    if (a.loss_hist) a.loss_hist[sv.epoch] = L;
+                    if (!isfinite(L)) atomicOr(a.status, ST_NONFINITE);
+                    sv.sse = 0.0;
+                    sv.step = 0;
+                    ++sv.epoch;
+                }
+            }
+        }
+        __syncwarp();
+    };
     for (int e = 0; e < a.epochs; ++e) {
-        sse_epoch = 0.0;
-        for (int64_t b0 = 0; b0 < a.n; b0 += mbs, ++step) {
-            const int64_t m = min(mbs, a.n - b0);
-            const bool epoch_end = b0 + mbs >= a.n;
-            const float c = a.loss_mean ? 1.0f / (float)m : 1.0f;
-            const int64_t r0 = b0 + (m * g) / G, r1 = b0 + (m * (g + 1)) / G;
-            long long *acc = a.acc + (size_t)((a.rot + step) % 3) * P1;
-            long long *acc_clear = a.acc + (size_t)((a.rot + step + 2) % 3) * P1;
+        int64_t b0 = 0;
+        for (int64_t st = 0; st < nsteps; ++st, b0 += mbs) {
+            const bool epoch_end = st == nsteps - 1;
+            const float c = a.loss_mean ? 1.0f / (float)(epoch_end ? a.n - b0 : mbs) : 1.0f;
+            const int64_t r0 = b0 + sv.lo[epoch_end], r1 = b0 + sv.hi[epoch_end];
+            long long *acc = a.acc + (size_t)rot * P1;
+            long long *acc_clear = a.acc + (size_t)(rot == 0 ? 2 : rot - 1) * P1;   // two steps ahead
+            rot = rot == 2 ? 0 : rot + 1;
 
             // ---- forward + backward over this block's rows of the step
             eng.load_weights(Wm);
-            if (resident) {
-                if (r1 > r0) eng.rows(Xs, ys, (int)(r1 - r0), c, zx);
+            if (resident || ahead) {
+                if (ahead) {
+                    cp_async_wait_all();
+                    __syncthreads();
+                }
+                if (r1 > r0) eng.rows(Xs + at * DP, ys + at, (int)(r1 - r0), c, zx);
+                if (ahead && (!epoch_end || e + 1 < a.epochs)) {
+                    // the next step's rows, to the other buffer (last read a step ago)
+                    at ^= CAP;
+                    const int64_t nb = epoch_end ? 0 : b0 + mbs;
+                    const int last = epoch_end ? nsteps == 1 : st + 2 == nsteps;
+                    const int64_t l = sv.lo[last], h = sv.hi[last];
+                    if (h > l) stage(nb + l, (int)(h - l), at);
+                }
             } else {
                 for (int64_t cs = r0; cs < r1; cs += CAP) {
                     const int cn = (int)min((int64_t)CAP, r1 - cs);
                     __syncthreads();
-                    stage(cs, cn);
+                    stage(cs, cn, 0);
                     cp_async_wait_all();
                     __syncthreads();
                     eng.rows(Xs, ys, cn, c, zx);
@@ -168,7 +245,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
             }
 
             // ---- block partial, in fixed point, into the global accumulator
-            eng.write_group(gpart, s_red);
+            eng.write_group(gpart, G == 1 ? s_ring[ring] : s_red);
             __syncthreads();
             if (G == 1) {
                 // A single block holds the whole step: its partial is the sum.  The
@@ -178,17 +255,27 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
                 const bool want_gn = a.gnorm_hist && epoch_end;
                 double gn = 0.0;
                 int bad = 0;
-                for (int p = tid; p < P; p += FNT) {
-                    float s = gpart[p];
+                for (int base = tid; base < P; base += 4 * FNT) {
+                    float v[4];   // four parameters in flight a thread
 #pragma unroll
-                    for (int q = 1; q < NG; ++q) s += gpart[q * P + p];
-                    const float v = s * gup;
-                    if (!(fabsf(v) < 4.0e18f)) bad = 1;
-                    // = (float)llrint(v) * 2^-gshift: below 2^23 both round v to the
-                    // same integer, above it v already is one (no 64-bit conversion)
-                    const float gsum = rintf(v) * gscale;
-                    Wm[p] -= a.lr * gsum;
-                    if (want_gn) gn = fma((double)gsum, (double)gsum, gn);
+                    for (int u = 0; u < 4; ++u) {
+                        const int p = min(base + u * FNT, P - 1);
+                        v[u] = gpart[p];
+#pragma unroll
+                        for (int q = 1; q < NG; ++q) v[u] += gpart[q * P + p];
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int p = base + u * FNT;
+                        if (p >= P) break;
+                        v[u] *= gup;
+                        if (!(fabsf(v[u]) < 4.0e18f)) bad = 1;
+                        // = (float)llrint(v) * 2^-gshift: below 2^23 both round v to the
+                        // same integer, above it v already is one (no 64-bit conversion)
+                        const float gsum = rintf(v[u]) * gscale;
+                        Wm[p] -= a.lr * gsum;
+                        if (want_gn) gn = fma((double)gsum, (double)gsum, gn);
+                    }
                 }
                 if (bad) atomicOr(a.status, ST_NONFINITE);
                 if (want_gn) {
@@ -196,24 +283,17 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
                     if ((tid & 31) == 0) s_gn[tid >> 5] = gn;
                 }
                 __syncthreads();
-                if (tid == 0) {
-                    double t = 0.0;
-                    for (int q = 0; q < NG; ++q) t += s_red[q];
-                    const double v = t * 4294967296.0;
-                    if (!(v < 4.0e18)) atomicOr(a.status, ST_NONFINITE);
-                    sse_epoch += (double)__double2ll_rn(v) * (1.0 / 4294967296.0);
-                    if (epoch_end) {
-                        const double L = 0.5 * sse_epoch * Cl;
-                        if (a.loss_hist) a.loss_hist[e] = L;
-                        if (!isfinite(L)) atomicOr(a.status, ST_NONFINITE);
-                        if (want_gn) {
-                            double u = 0.0;
-                            for (int q = 0; q < RE_NW; ++q) u += s_gn[q];
-                            a.gnorm_hist[e] = sqrt(u);
-                        }
-                    }
+                if (want_gn && tid == 0) {
+                    double u = 0.0;
+                    for (int q = 0; q < RE_NW; ++q) u += s_gn[q];
+                    a.gnorm_hist[e] = sqrt(u);
                 }
-                __syncthreads();
+                // The loss takes a dozen dependent FP64 operations (1,200 cycles in one
+                // thread): RING steps' at a time, a lane each, while the next step runs.
+                if ((++ring & (RING - 1)) == 0) {
+                    if (tid < 32) finish_steps(ring - RING, RING);
+                    if (ring == 2 * RING) ring = 0;
+                }
                 continue;
             }
             // Each of the G block partials stays below 2^63 / G in magnitude, so
@@ -227,7 +307,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
                 for (int q = 1; q < NG; ++q) s += gpart[q * P + p];
                 const float v = s * gup;
                 if (!(fabsf(v) < lim)) bad = 1;   // out of range or NaN
-                red_add(acc + p, __float2ll_rn(v));
+                red_add(acc + p, float_to_fixed(v));
             }
             if (tid == 0) {
                 double t = 0.0;
@@ -245,19 +325,19 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
             const bool want_gn = g == 0 && a.gnorm_hist && epoch_end;
             double gn = 0.0;
             // the gradient and the squared error (entry P) in one round trip
-            for (int base = 0; base < P1; base += 12 * FNT) {
-                long long v[12];  // twelve loads in flight per thread: one round trip up to P = 3071
+            for (int base = 0; base < P1; base += 16 * FNT) {
+                long long v[16];  // sixteen loads in flight per thread: one round trip up to P = 4095
 #pragma unroll
-                for (int r = 0; r < 12; ++r) {
+                for (int r = 0; r < 16; ++r) {
                     const int p = base + r * FNT + tid;
                     v[r] = (p < P1) ? __ldcg(acc + p) : 0ll;
                 }
 #pragma unroll
-                for (int r = 0; r < 12; ++r) {
+                for (int r = 0; r < 16; ++r) {
                     const int p = base + r * FNT + tid;
                     if (p == P) s_sse = v[r];
                     if (p < P) {
-                        const float gsum = (float)v[r] * gscale;
+                        const float gsum = fixed_to_float(v[r]) * gscale;
                         Wm[p] -= a.lr * gsum;
                         if (want_gn) gn = fma((double)gsum, (double)gsum, gn);
                     }
@@ -272,9 +352,11 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
                 }
                 __syncthreads();
                 if (tid == 0) {
-                    sse_epoch += (double)s_sse * (1.0 / 4294967296.0);
+                    sv.fix += s_sse;   // at most n 2^32 and a rounding a block and step: exact
                     if (epoch_end) {
-                        const double L = 0.5 * sse_epoch * Cl;
+                        const double Cl = a.loss_mean ? 1.0 / (double)a.n : 1.0;
+                        const double L = 0.5 * ((double)sv.fix * (1.0 / 4294967296.0)) * Cl;
+                        sv.fix = 0;
                         if (a.loss_hist) a.loss_hist[e] = L;
                         if (!isfinite(L)) atomicOr(a.status, ST_NONFINITE);
                         if (want_gn) {
@@ -288,6 +370,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
             __syncthreads();
         }
     }
+    if (G == 1 && tid < 32 && (ring & (RING - 1)) != 0) finish_steps(ring & ~(RING - 1), ring & (RING - 1));
     if (g == 0)
         for (int p = tid; p < P; p += FNT) a.params[p] = Wm[p];
 }
@@ -377,6 +460,14 @@ int blocks_per_sm(void *fn, size_t smem, cudaError_t *err) {
     return per_sm;
 }
 
+// Rows a block takes unless the caller says: 16 where that makes at most one
+// block an SM, else 32.  A block's turn of 16 rows (33-100-1) is 2 us, its share
+// of the cross-block sum and the barrier 5 us whatever its rows: mini-batches of
+// 1000 rows take 181 us for 20 steps with 16 rows a block, 222 with 32 and 187
+// with 8; 4096 rows in one step 15.1 us with 16 and 14.6 with 32.  Steps of at
+// most 32 rows stay one block, which needs neither sum nor barrier.
+int auto_rows(int64_t mbs) { return mbs > 32 && mbs <= 16 * (int64_t)device_sm_count() ? 16 : 32; }
+
 }  // namespace
 
 bool fused_supported(int D, int H) {
@@ -406,13 +497,13 @@ cudaError_t fused_train(int act, int D, int H, int64_t n, const float *X, const 
     Choice ch;
     if (!choose(act, D, H, &ch)) return cudaErrorInvalidValue;
     const int64_t mbs = (mb <= 0 || mb >= n) ? n : mb;
-    if (rows_per_block < 1) rows_per_block = 32;
+    if (rows_per_block < 1) rows_per_block = auto_rows(mbs);
     int64_t G = cdiv(mbs > 0 ? mbs : 1, rows_per_block);
     if (G > GMAX) G = GMAX;
     if (G < 1) G = 1;
     // Shared memory depends on whether the rows stay resident.
     bool resident = (mbs == n) && cdiv(mbs, G) <= RESIDENT;
-    size_t smem = choice_smem(ch, D, H, resident ? RESIDENT : CAP);
+    size_t smem = choice_smem(ch, D, H, resident ? RESIDENT : 2 * CAP);
     cudaError_t e;
     int per_sm = blocks_per_sm(ch.fn, smem, &e);
     if (e != cudaSuccess) return e;
@@ -421,7 +512,7 @@ cudaError_t fused_train(int act, int D, int H, int64_t n, const float *X, const 
     if (G > cap) {
         G = cap;
         resident = (mbs == n) && cdiv(mbs, G) <= RESIDENT;
-        smem = choice_smem(ch, D, H, resident ? RESIDENT : CAP);
+        smem = choice_smem(ch, D, H, resident ? RESIDENT : 2 * CAP);
         per_sm = blocks_per_sm(ch.fn, smem, &e);
         if (e != cudaSuccess) return e;
         if ((int64_t)per_sm * device_sm_count() < G) return cudaErrorInvalidConfiguration;
