@@ -593,7 +593,11 @@ cudaError_t forward_t(int act, int D, int H, int64_t n, const void *X, const voi
                       const void *w2, const void *b2, void *hid, void *o, const void *y, const void *dLdo,
                       double c, const PlainWork &w, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    if (act == MLP_ACT_TANH) hidden_act<T, TX, MLP_ACT_TANH>(D, H, n, X, W1, b1, w2, hid, w, st);
+    const int prec = sizeof(T) == 8 ? MLP_FP64 : (sizeof(TX) == 2 ? MLP_BF16 : MLP_FP32);
+    if (split_forward_takes(prec, D, H, n)) {
+        const cudaError_t e = split_forward(prec, act, D, H, n, X, W1, b1, w2, hid, w.z2part, st);
+        if (e != cudaSuccess) return e;
+    } else if (act == MLP_ACT_TANH) hidden_act<T, TX, MLP_ACT_TANH>(D, H, n, X, W1, b1, w2, hid, w, st);
     else hidden_act<T, TX, MLP_ACT_SIGMOID>(D, H, n, X, W1, b1, w2, hid, w, st);
     k_fwd_output<T><<<(unsigned)cdiv(n, 256), 256, 0, st>>>((int)cdiv(H, TJ), n, (const T *)w.z2part,
                                                             (const T *)b2, (T *)o, (const T *)y,

@@ -62,3 +62,60 @@ def test_training_steps_update_and_loss(n, D, H, mb, loss_mean):
     assert rel_err_norm(got, q.flat()) <= W_TOL
     np.testing.assert_allclose(host(lh), l_ref, rtol=1e-6)
     np.testing.assert_allclose(host(gh), g_ref, rtol=1e-4)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("n,D,H", [(6144, 1, 65), (6144, 33, 65), (6100, 47, 128), (3073, 48, 200), (1025, 64, 770),
+                                   (20001, 16, 129), (129, 49, 3072)])
+def test_tensor_core_forward(n, D, H, prec):
+    """The split forward (D <= 64, H > 64, at least 48 tiles): every K step,
+    remainders of rows and units, hid with and without 16-byte rows, at the
+    FP32 bar; hidden activations within the bound of an FP32 sum of D + 1 terms,
+    (D + 1) 2^-24 sum |x w|, and 1e-6 of their value for the activation (its
+    slope is at most 1)."""
+    import torch
+    from paper_1908_07847_gb300 import inputs as I
+    act = D % 2
+    X, _, W = problem(7300 + n + D, n, D, H)
+    if prec == "bf16":
+        X = I.bf16_round(X)
+        with Net(D, H, prec=B.MLP_BF16, act=act) as net:
+            net.set(W)
+            o = torch.zeros(n, device="cuda")
+            B.mlp_forward(net.h, dev(X).to(torch.bfloat16), n, o, stream())
+            got, hid = host(o), None
+    else:
+        t = [dev(np.asarray(a, np.float32)) for a in (X, *W)]
+        hd, o = torch.zeros((n, H), device="cuda"), torch.zeros(n, device="cuda")
+        nb = B.mlp_workspace_bytes(B.MLP_FP32, D, H, n)
+        ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+        B.mlp_forward_w(B.MLP_FP32, act, D, H, n, *t, hd, o, ws, nb, stream())
+        got, hid = host(o), host(hd)
+    h_ref, o_ref = oracle.forward(X, Params(*W), act)
+    assert rel_err_elem(got, o_ref) <= FWD_TOL
+    if hid is not None:
+        size = np.abs(X.astype(np.float64)) @ np.abs(W[0].astype(np.float64)).T + np.abs(W[1])
+        assert np.all(np.abs(hid - h_ref) <= (D + 1) * 2.0 ** -24 * size + 1e-6 * np.abs(h_ref))
+
+
+@pytest.mark.parametrize("where", ["x", "w"])
+def test_tensor_core_forward_of_values_outside_the_parts_range(where):
+    """Infinities, NaN, huge and tiny values in one row (or one unit's
+    weights): those tiles take plain FP32 multiply-adds, the others do not
+    notice.  An infinite input saturates its units as in 64 bits."""
+    import torch
+    n, D, H = 6400, 33, 130
+    X, _, W = problem(7400, n, D, H)
+    X[7, 3], X[200, 0], X[333, 1], X[500, 2], X[600, 5] = np.inf, -np.inf, 3.3e38, 1e-38, np.nan
+    if where == "w":
+        W[0][5, 4], W[0][129, 0] = 1e30, 1e-35
+    with Net(D, H) as net:
+        net.set(W)
+        o = torch.zeros(n, device="cuda")
+        B.mlp_forward(net.h, dev(X), n, o, stream())
+        got = host(o)
+    with np.errstate(all="ignore"):
+        _, ref = oracle.forward(X, Params(*W))
+    assert np.isnan(got[600]) and np.isnan(ref[600])
+    ok = np.arange(n) != 600
+    assert rel_err_elem(got[ok], ref[ok]) <= FWD_TOL
