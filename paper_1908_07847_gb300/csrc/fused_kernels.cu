@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     // kept here rather than in every thread's registers (the row engine fills them)
     __shared__ struct {
         int64_t lo[2], hi[2];   // this block's rows of a full step [0] and of the last, ragged one [1]
+        float c[2];             // and the scale of their output deltas
         double sse;             // one block: squared error of the epoch so far
         long long fix;          // several: the same as the sum of the steps' fixed-point values
         int64_t step;           // one block: of the epoch, the next step to finish
@@ -125,6 +126,8 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
         sv.hi[0] = (mbs * (g + 1)) / G;
         sv.lo[1] = (ml * g) / G;
         sv.hi[1] = (ml * (g + 1)) / G;
+        sv.c[0] = a.loss_mean ? 1.0f / (float)mbs : 1.0f;
+        sv.c[1] = a.loss_mean ? 1.0f / (float)ml : 1.0f;
         sv.sse = 0.0;
         sv.fix = 0;
         sv.step = 0;
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
         int64_t b0 = 0;
         for (int64_t st = 0; st < nsteps; ++st, b0 += mbs) {
             const bool epoch_end = st == nsteps - 1;
-            const float c = a.loss_mean ? 1.0f / (float)(epoch_end ? a.n - b0 : mbs) : 1.0f;
+            const float c = sv.c[epoch_end];
             const int64_t r0 = b0 + sv.lo[epoch_end], r1 = b0 + sv.hi[epoch_end];
             long long *acc = a.acc + (size_t)rot * P1;
             long long *acc_clear = a.acc + (size_t)(rot == 0 ? 2 : rot - 1) * P1;   // two steps ahead

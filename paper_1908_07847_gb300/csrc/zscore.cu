@@ -14,7 +14,7 @@
 // rows at a time are first added in FP32 with their rounding errors kept
 // (Knuth's two-sum; Ogita, Rump and Oishi, "Accurate sum and dot product", 2005,
 // and the fused multiply-add's exact product error for the squares), and only the
-// group's sum and error go to FP64: 71 us (5.5 TB/s) and 211 us a pass.
+// group's sum and error go to FP64: 71 and about 150 us a pass.
 // The errors add up to 2^-24 of the sum and are themselves kept to 24 bits, so a
 // group is off by about 2^-48 of one element, below the rounding of the FP64
 // accumulator it is added to.  Groups whose values leave FP32's safe range
@@ -43,6 +43,12 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
 }
 
+template <int N>
+__device__ __forceinline__ void load_group(float (&v)[N], const float *p, int64_t step) {
+#pragma unroll
+    for (int u = 0; u < N; ++u) v[u] = __ldg(p + u * step);
+}
+
 // The same rows element by element in FP64 (kept out of line: inlined, the
 // compiler ran its FP64 instructions for every group).
 template <int P>
@@ -58,10 +64,8 @@ __device__ __noinline__ double add_fp64(double acc, const float *p, int64_t step
 // acc += sum of v[u] (P = 1) or of (v[u] - c)^2 (P = 2, c = chi + clo up to
 // 2^-49): a tree of two-sums over the group, the errors added in a fixed order.
 template <int P, int N>
-__device__ __forceinline__ void add_group(double &acc, const float *p, int64_t step, double c, float chi, float clo) {
-    float v[N];
-#pragma unroll
-    for (int u = 0; u < N; ++u) v[u] = __ldg(p + u * step);
+__device__ __forceinline__ void add_group(double &acc, const float (&v)[N], const float *p, int64_t step, double c,
+                                          float chi, float clo) {
     float x[N];
     float m = 0.f, lo = 0.f;   // m: the largest |value| or |deviation|
 #pragma unroll
@@ -120,8 +124,27 @@ __global__ void __launch_bounds__(ZT) k_colsum(const float *__restrict__ X, int6
             int64_t i = r0 + rl;
             const float *p = X + i * D + j;
             const int64_t step = (int64_t)RL * D;
-            for (; i + (ZG - 1) * RL < r1; i += ZG * RL, p += ZG * step) add_group<P, ZG>(acc, p, step, c, chi, clo);
-            for (; i + 3 * RL < r1; i += 4 * RL, p += 4 * step) add_group<P, 4>(acc, p, step, c, chi, clo);
+            // a group's loads are in flight while the one before is added up (without
+            // that the second pass waits for memory and takes 211 us)
+            float v[ZG];
+            bool more = i + (ZG - 1) * RL < r1;
+            if (more) load_group<ZG>(v, p, step);
+            while (more) {
+                const float *cur = p;
+                float w[ZG];
+                i += ZG * RL;
+                p += ZG * step;
+                more = i + (ZG - 1) * RL < r1;
+                load_group<ZG>(w, more ? p : cur, step);
+                add_group<P, ZG>(acc, v, cur, step, c, chi, clo);
+#pragma unroll
+                for (int u = 0; u < ZG; ++u) v[u] = w[u];
+            }
+            for (; i + 3 * RL < r1; i += 4 * RL, p += 4 * step) {
+                float v4[4];
+                load_group<4>(v4, p, step);
+                add_group<P, 4>(acc, v4, p, step, c, chi, clo);
+            }
             for (; i < r1; i += RL, p += step) {
                 const double d = (double)*p - c;
                 acc += P == 2 ? d * d : d;
