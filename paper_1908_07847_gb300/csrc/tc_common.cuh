@@ -79,6 +79,14 @@ __device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t a, uint64_t b,
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
+// The same with A in tensor memory (lane = row of A, two consecutive K values
+// in bf16 a column).
+__device__ __forceinline__ void mma_bf16_ta(uint32_t dtmem, uint32_t atmem, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(dtmem),
+        "r"(atmem), "l"(b), "r"(idesc), "r"(acc));
+}
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
@@ -188,6 +196,14 @@ __device__ __forceinline__ float dot2_bf16(uint32_t a, uint32_t b, float acc) {
         : "=f"(d)
         : "r"(a), "r"(b), "f"(acc));
     return d;
+}
+// acc0 += a.lo b.lo, acc1 += a.hi b.lo: two rows' shares of a product with one
+// weight, accumulated in FP32.
+__device__ __forceinline__ void fma_rows(uint32_t a, uint32_t b, float &acc0, float &acc1) {
+    asm("{\n\t.reg .b16 al, ah, bl, bh;\n\tmov.b32 {al, ah}, %2;\n\tmov.b32 {bl, bh}, %3;\n\t"
+        "fma.rn.f32.bf16 %0, al, bl, %0;\n\tfma.rn.f32.bf16 %1, ah, bl, %1;\n\t}"
+        : "+f"(acc0), "+f"(acc1)
+        : "r"(a), "r"(b));
 }
 // sigmoid of a pair given half its argument: 1/2 + tanh(x/2)/2.
 __device__ __forceinline__ uint32_t sigmoid_half_bf2(uint32_t xhalf) { return hfma2(tanh_bf2(xhalf), BF2_HALF, BF2_HALF); }
