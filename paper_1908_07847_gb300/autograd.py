@@ -10,6 +10,8 @@ differences.  Marshalling only: both directions run in the CUDA library.
 """
 from __future__ import annotations
 
+import functools
+
 import torch
 
 from . import binding as B
@@ -17,8 +19,15 @@ from . import binding as B
 _PREC = {torch.float32: B.MLP_FP32, torch.float64: B.MLP_FP64}
 
 
+@functools.lru_cache(maxsize=256)
+def _workspace_bytes(prec, D, H, n, index):
+    with torch.cuda.device(index):
+        return B.mlp_workspace_bytes(prec, D, H, n)
+
+
 def _workspace(prec, D, H, n, device):
-    nbytes = B.mlp_workspace_bytes(prec, D, H, n)
+    # the size depends on the shape and the device alone
+    nbytes = _workspace_bytes(prec, D, H, n, device.index)
     # torch's allocator returns blocks aligned to at least 512 bytes.
     return torch.empty(max(nbytes, 1), dtype=torch.uint8, device=device), nbytes
 

@@ -206,7 +206,7 @@ cudaError_t plain_forward(int prec, int act, int D, int H, int64_t n, const void
 // The forward products on the tensor cores at FP32 accuracy (split_forward.cu):
 // whether a shape goes there, and the launch (hid may be NULL; z2part as
 // PlainWork's, one row of n for every 64 units).
-bool split_forward_takes(int prec, int D, int H, int64_t n);
+bool split_forward_takes(int prec, int D, int H, int64_t n, bool hid);
 cudaError_t split_forward(int prec, int act, int D, int H, int64_t n, const void *X, const void *W1, const void *b1,
                           const void *w2, void *hid, void *z2part, cudaStream_t st);
 

@@ -38,39 +38,43 @@ __device__ __forceinline__ void lds(T (&v)[N], const T *p) {
 // k < ks; src rows are ld apart, dst rows st = 4 mod 32 apart.  A warp takes 4
 // rows x 8 inputs: whole 32-byte sectors of the rows, and all 32 banks of the
 // transposed side.  Eight such patches are in flight a warp (one at a time, the
-// loads' latency took longer than the products).
+// loads' latency took longer than the products); a warp keeps its rows, so that
+// no index is divided.
 template <int TR, typename T, typename TX>
 __device__ __forceinline__ void stage_t(T *dst, int st, const TX *src, int64_t ld, int64_t nr, int ks) {
-    const int lane = threadIdx.x & 31, kq = (ks + 7) >> 3, tot = (TR / 4) * kq;
-    for (int w0 = threadIdx.x >> 5; w0 < tot; w0 += NTH / 32 * 8) {
-        T v[8];
+    constexpr int R = TR >= 32 ? TR / 32 : 1, KB = 8 / R;   // patches of rows and of inputs in flight
+    const int lane = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * 4 + (lane >> 3);
+    if (TR < 32 && r0 >= TR) return;
+    for (int k0 = lane & 7; k0 < ks; k0 += 8 * KB) {
+        T v[KB][R];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int w = w0 + u * (NTH / 32), rb = w / kq, k = (w - rb * kq) * 8 + (lane & 7), r = rb * 4 + (lane >> 3);
-            v[u] = (w < tot && k < ks && r < nr) ? ldx<T, TX>(src, r * ld + k) : T(0);
-        }
+        for (int c = 0; c < KB; ++c)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int w = w0 + u * (NTH / 32), rb = w / kq, k = (w - rb * kq) * 8 + (lane & 7), r = rb * 4 + (lane >> 3);
-            if (w < tot && k < ks) dst[k * st + r] = v[u];
-        }
+            for (int i = 0; i < R; ++i) {
+                const int k = k0 + 8 * c, r = r0 + 32 * i;
+                v[c][i] = (k < ks && r < nr) ? ldx<T, TX>(src, r * ld + k) : T(0);
+            }
+#pragma unroll
+        for (int c = 0; c < KB; ++c)
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+                if (k0 + 8 * c < ks) dst[(k0 + 8 * c) * st + r0 + 32 * i] = v[c][i];
     }
 }
 
 // The same as asynchronous copies (T on both sides), waited for later.
 template <int TR, typename T>
 __device__ __forceinline__ void stage_t_async(T *dst, int st, const T *src, int64_t ld, int64_t nr, int ks) {
-    const int lane = threadIdx.x & 31, kq = (ks + 7) >> 3, tot = (TR / 4) * kq;
-#pragma unroll 4
-    for (int w = threadIdx.x >> 5; w < tot; w += NTH / 32) {
-        const int rb = w / kq, k = (w - rb * kq) * 8 + (lane & 7), r = rb * 4 + (lane >> 3);
-        if (k < ks) {
-            const unsigned d = (unsigned)__cvta_generic_to_shared(dst + k * st + r);
-            const T *g = src + (r < nr ? r : 0) * ld + k;
-            const int bytes = r < nr ? (int)sizeof(T) : 0;   // the rest is zero-filled
-            asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(g), "n"(sizeof(T)), "r"(bytes)
+    const int lane = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * 4 + (lane >> 3);
+#pragma unroll
+    for (int i = 0; i < TR / 32; ++i) {
+        const int r = r0 + 32 * i;
+        const T *g = src + (r < nr ? r : 0) * ld;
+        const int bytes = r < nr ? (int)sizeof(T) : 0;   // the rest is zero-filled
+        unsigned d = (unsigned)__cvta_generic_to_shared(dst + (lane & 7) * st + r);
+        for (int k = lane & 7; k < ks; k += 8, d += 8 * st * (unsigned)sizeof(T))
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(g + k), "n"(sizeof(T)), "r"(bytes)
                          : "memory");
-        }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -88,7 +92,9 @@ __device__ __forceinline__ void stage_t_async(T *dst, int st, const T *src, int6
 // the SM's FMA pipes), where 4 x 4 tiles with four-byte loads were held by
 // shared memory.  RPT falls to 4, 2 or 1 where the grid would not fill the
 // device (forward_t).  The order of every sum is that of one pass over the
-// inputs and of a fixed tree over the units, whatever RPT is.
+// inputs and of a fixed tree over the units, whatever RPT is.  Whole forward calls,
+// 4 x 4 tiles and now: 83-166, 140024 rows 233 and 146 us; 84-37, 17620 rows 15.4
+// and 12.1; 31-98, 230 rows 7.1 and 5.7; FP64 17-809, 1234 rows 129 and 89.
 template <typename T, typename TX, int ACT, int RPT>
 __global__ void __launch_bounds__(NTH) k_fwd_hidden(int D, int H, int64_t n, int tpb, const TX *__restrict__ X,
                                                     const T *__restrict__ W1, const T *__restrict__ b1,
@@ -228,7 +234,11 @@ __global__ void k_d2_upstream(int64_t n, const T *__restrict__ o, const T *__res
 // A thread holds 8 units x 4 inputs (three 16-byte loads for 32 multiply-adds
 // a row); the tile's inputs are cut into quads, so 33 inputs cost 36 and not
 // 64.  The 8 x kq thread tiles leave room for RS row subsets (2 to 32), each
-// summing every RS-th row; the subsets are added in order at the end.
+// summing every RS-th row; the subsets are added in a fixed tree at the end.  The
+// next slice's values load while the present one is summed (a slice's loads one
+// after the other took 10,000 cycles).  Whole gradient calls, 4 x 4 tiles of 64
+// inputs and now: 83-458, 105224 rows 1510 and 765 us; 65-285, 163 rows 18.9 and
+// 14.6; FP64 11-24, 1018 rows 72 and 35.
 constexpr int GR = 32;   // rows staged at a time
 
 template <typename T, typename TX, int ACT>
@@ -248,7 +258,9 @@ __global__ void __launch_bounds__(NTH) k_bwd_grad(int D, int H, int64_t n, int64
     const int kn = min(64, D - k0), kq = (kn + 3) >> 2;   // inputs of this tile, in quads
     const int RS = NTH / (8 * kq);                        // row subsets
     const int rs = tid / (8 * kq), t = tid - rs * 8 * kq;
-    const int u8 = (t & 7) * 8, k4 = (t >> 3) * 4;        // this thread's units and inputs
+    // this thread's units and inputs; neighbouring lanes along the inputs: few
+    // distinct words of Ds a load, consecutive ones of Xs, and nearby stores
+    const int u8 = (t / kq) * 8, k4 = (t - (t / kq) * kq) * 4;
     T acc[8][4];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
@@ -302,25 +314,28 @@ __global__ void __launch_bounds__(NTH) k_bwd_grad(int D, int H, int64_t n, int64
         }
     }
     T *pc = part + c * P;
-    // the row subsets in order, through shared memory four units at a time
-    for (int q = 1; q < RS; ++q) {
-        __syncthreads();
-        T *buf = &Ds[0][0];   // 16 values of each of a subset's 8 kq <= 128 tiles
+    // the row subsets by halving, through shared memory four units at a time (one
+    // after the other, 16 subsets of a narrow tile took 60 barriers)
+    for (int m = RS; m > 1;) {
+        const int h = (m + 1) / 2;
+        T *buf = &Ds[0][0];   // 16 values of each of at most 128 threads' tiles
+        const int w = 8 * kq * (m - h);
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-            if (rs == q)
+            __syncthreads();
+            if (rs >= h && rs < m)
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) buf[(i * 4 + kk) * (8 * kq) + t] = acc[4 * half + i][kk];
+                    for (int kk = 0; kk < 4; ++kk) buf[(i * 4 + kk) * w + (rs - h) * 8 * kq + t] = acc[4 * half + i][kk];
             __syncthreads();
-            if (rs == 0)
+            if (rs < m - h)
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) acc[4 * half + i][kk] += buf[(i * 4 + kk) * (8 * kq) + t];
-            __syncthreads();
+                    for (int kk = 0; kk < 4; ++kk) acc[4 * half + i][kk] += buf[(i * 4 + kk) * w + rs * 8 * kq + t];
         }
+        m = h;
     }
     if (rs == 0) {
 #pragma unroll
@@ -580,10 +595,12 @@ void hidden_act(int D, int H, int64_t n, const void *X, const void *W1, const vo
         // small blocks spread evenly
         launch_hidden<T, TX, ACT, 1>(D, H, n, X, W1, b1, w2, hid, w, sms, st);
     } else {
-        // the largest tile that still gives two blocks an SM
-        const int64_t tj = cdiv(H, TJ), want = 2 * (int64_t)sms;
-        if (cdiv(n, 128) * tj >= want) launch_hidden<T, TX, ACT, 8>(D, H, n, X, W1, b1, w2, hid, w, sms, st);
-        else if (cdiv(n, 64) * tj >= want) launch_hidden<T, TX, ACT, 4>(D, H, n, X, W1, b1, w2, hid, w, sms, st);
+        // 128-row tiles where they still give two blocks an SM, 64-row tiles down
+        // to one (84-37, 17620 rows: 16.9 us with 276 tiles of 64 rows, 21.0 with
+        // 551 of 32; 80-149, 1043 rows: 13.4 with 51 and 10.5 with 99)
+        const int64_t tj = cdiv(H, TJ);
+        if (cdiv(n, 128) * tj >= 2 * (int64_t)sms) launch_hidden<T, TX, ACT, 8>(D, H, n, X, W1, b1, w2, hid, w, sms, st);
+        else if (cdiv(n, 64) * tj >= sms) launch_hidden<T, TX, ACT, 4>(D, H, n, X, W1, b1, w2, hid, w, sms, st);
         else launch_hidden<T, TX, ACT, 2>(D, H, n, X, W1, b1, w2, hid, w, sms, st);
     }
 }
@@ -594,7 +611,7 @@ cudaError_t forward_t(int act, int D, int H, int64_t n, const void *X, const voi
                       double c, const PlainWork &w, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     const int prec = sizeof(T) == 8 ? MLP_FP64 : (sizeof(TX) == 2 ? MLP_BF16 : MLP_FP32);
-    if (split_forward_takes(prec, D, H, n)) {
+    if (split_forward_takes(prec, D, H, n, hid != nullptr)) {
         const cudaError_t e = split_forward(prec, act, D, H, n, X, W1, b1, w2, hid, w.z2part, st);
         if (e != cudaSuccess) return e;
     } else if (act == MLP_ACT_TANH) hidden_act<T, TX, MLP_ACT_TANH>(D, H, n, X, W1, b1, w2, hid, w, st);

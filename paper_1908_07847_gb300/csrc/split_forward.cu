@@ -262,14 +262,21 @@ cudaError_t launch(int D, int H, int64_t n, const void *X, const void *W1, const
 
 }  // namespace
 
-// Up to 64 inputs (what the parts' tiles hold), more than one tile of 64 units,
-// and enough tiles of 128 x 128 to be worth a tile's latency.  At 64 tiles
-// (whole forward calls, against FP32 multiply-adds): 33-512, 2048 rows 10.3 and
-// 11.8 us; 64-1000, 1024 rows 12.0 and 15.1; 33-96, 8192 rows 10.5 and 11.8;
-// bf16 48-2048, 512 rows 9.8 and 14.2; below 32 tiles the two are equal or the
-// multiply-adds win.
-bool split_forward_takes(int prec, int D, int H, int64_t n) {
-    return prec != MLP_FP64 && D <= 64 && H > 64 && ((n + SR - 1) / SR) * ((H + SU - 1) / SU) >= 48;
+// From 12 to 64 inputs (what the parts' tiles hold), more than one tile of 64
+// units, and enough tiles of 128 x 128.  Whole forward calls, FP32 multiply-adds
+// against this: 12-512 4096 rows (128 tiles) 8.4 and 8.4 us, 8192 rows 12.3 and
+// 9.8; 33-512 2048 rows 7.4 and 10.4, 4096 rows 11.2 and 10.5; 33-96 16384 rows
+// 11.2 and 10.7; bf16 48-2048 1024 rows 13.7 and 9.9.  Storing the activations, a
+// row a thread, costs more here, the more so the fewer the inputs: 16-512 65536
+// rows 69.3 and 74.0; 33-512 4096 rows 11.3 and 13.2, 8192 rows 17.8 and 17.9,
+// 65536 rows 95.4 and 91.7; 64-512 4096 rows 15.6 and 14.6.  Rows of hid that do
+// not start on 16 bytes are stored four bytes at a time (56-433, 2060 rows: a
+// gradient call 36 us, 28 with multiply-adds).
+bool split_forward_takes(int prec, int D, int H, int64_t n, bool hid) {
+    if (prec == MLP_FP64 || D < 12 || D > 64 || H <= 64) return false;
+    const int64_t tiles = ((n + SR - 1) / SR) * ((H + SU - 1) / SU);
+    if (hid && ((H & 3) != 0 || D <= 32 || D * tiles < 8192)) return false;
+    return tiles >= 128;
 }
 
 cudaError_t split_forward(int prec, int act, int D, int H, int64_t n, const void *X, const void *W1, const void *b1,
