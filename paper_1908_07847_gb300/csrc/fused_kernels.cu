@@ -120,14 +120,16 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     const bool ahead = !resident && rows_max <= CAP;
     const int xcap = resident ? RESIDENT : 2 * CAP;
     const int64_t nsteps = cdiv(a.n, mbs);
-    if (tid == 0) {   // once: a 64-bit division costs hundreds of cycles
-        const int64_t ml = a.n - (nsteps - 1) * mbs;
-        sv.lo[0] = (mbs * g) / G;
-        sv.hi[0] = (mbs * (g + 1)) / G;
-        sv.lo[1] = (ml * g) / G;
-        sv.hi[1] = (ml * (g + 1)) / G;
-        sv.c[0] = a.loss_mean ? 1.0f / (float)mbs : 1.0f;
-        sv.c[1] = a.loss_mean ? 1.0f / (float)ml : 1.0f;
+    // Once, a thread each (the rows' copies wait for them): a 64-bit division
+    // takes hundreds of cycles, a 32-bit one does for most steps.
+    if (tid < 4) {
+        const int64_t m = tid < 2 ? mbs : a.n - (nsteps - 1) * mbs, x = m * (g + (tid & 1));
+        const int64_t v = x <= INT32_MAX ? (int64_t)((uint32_t)x / (uint32_t)G) : x / G;
+        if (tid & 1) sv.hi[tid >> 1] = v;
+        else sv.lo[tid >> 1] = v;
+        if (!(tid & 1)) sv.c[tid >> 1] = a.loss_mean ? 1.0f / (float)m : 1.0f;
+    }
+    if (tid == 4) {
         sv.sse = 0.0;
         sv.fix = 0;
         sv.step = 0;
