@@ -54,6 +54,16 @@ constexpr int TR = 128;           // rows per tile
 constexpr int SUB = 64;           // rows of a half tile
 constexpr int HMAX = 256;
 constexpr int NSTAGE = 6;         // X tiles in shared memory
+constexpr int NZ1 = 3;            // Z1 / d1 buffers in tensor memory
+// Barriers of the two hand-overs between MMAs and epilogue.  A parity wait sees
+// one phase back, so a barrier must not complete twice before its waiter has
+// looked.  One barrier a group would: the forward of half tile s only waits for
+// the buffer's last reader, s - 3, a half of the other group, so s - 2 and s can
+// both be done while a thread of their group still looks for s - 2.  Here the
+// next phase of a barrier needs the same buffer again, hence everyone's work on
+// the one before.
+constexpr int NZ1F = 2 * NZ1;     // forward done: a group and buffer
+constexpr int NDF = NZ1;          // d1 written: a buffer
 constexpr int NEPI = 16;          // epilogue warps: two groups of 4 lane quarters x 2 row halves
 constexpr int NT = (2 + NEPI) * 32;  // threads: forward warp, gradient and TMA warp, epilogue warps
 constexpr uint32_t NEPI_T = NEPI * 32;
@@ -112,14 +122,18 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
     float *w2s = (float *)(sm + SM_W2);
     const uint32_t bar0 = sb + SM_BAR;
     // TMA -> MMA: FULL (a stage); gradient MMA -> TMA: EMPTY (a stage); forward
-    // MMA -> epilogue: Z1F (a group); epilogue -> gradient MMA: DF (a group's d1
-    // written); gradient MMA -> forward: GD (a Z1 buffer read), -> epilogue:
-    // EPOCH; epilogue -> forward: W (weights updated); among epilogue threads: EPI
-    // (a group), EPIA (both).
-    const uint32_t BAR_FULL = bar0, BAR_EMPTY = BAR_FULL + 8 * NSTAGE, BAR_Z1F = BAR_EMPTY + 8 * NSTAGE,
-                   BAR_GD = BAR_Z1F + 16, BAR_DF = BAR_GD + 24, BAR_EPOCH = BAR_DF + 16, BAR_W = BAR_EPOCH + 8,
-                   BAR_EPI = BAR_W + 8, BAR_EPIA = BAR_EPI + 16, BAR_DRAIN = BAR_EPIA + 8;
-    constexpr int NBAR = 2 * NSTAGE + 14;
+    // MMA -> epilogue: Z1F (a group and Z1 buffer); epilogue -> gradient MMA: DF (a
+    // buffer's d1 written); gradient MMA -> forward: GD (a buffer read), ->
+    // epilogue: EPOCH; epilogue -> forward: W (weights updated); among epilogue
+    // threads: EPI (a group), EPIA (both).
+    constexpr int I_EMPTY = NSTAGE, I_Z1F = I_EMPTY + NSTAGE, I_GD = I_Z1F + NZ1F, I_DF = I_GD + NZ1,
+                  I_EPOCH = I_DF + NDF, I_W = I_EPOCH + 1, I_EPI = I_W + 1, I_EPIA = I_EPI + 2, I_DRAIN = I_EPIA + 1,
+                  NBAR = I_DRAIN + 2;
+    static_assert(8 * NBAR <= SM_MISC - SM_BAR, "barriers");
+    const uint32_t BAR_FULL = bar0, BAR_EMPTY = bar0 + 8 * I_EMPTY, BAR_Z1F = bar0 + 8 * I_Z1F,
+                   BAR_GD = bar0 + 8 * I_GD, BAR_DF = bar0 + 8 * I_DF, BAR_EPOCH = bar0 + 8 * I_EPOCH,
+                   BAR_W = bar0 + 8 * I_W, BAR_EPI = bar0 + 8 * I_EPI, BAR_EPIA = bar0 + 8 * I_EPIA,
+                   BAR_DRAIN = bar0 + 8 * I_DRAIN;
     uint32_t *tmem_slot = (uint32_t *)(sm + SM_MISC);
     volatile int *abort = (volatile int *)(sm + SM_MISC + 16);
     float *red = (float *)(sm + SM_MISC + 64);     // 4 warps x (sse, gb2)
@@ -134,10 +148,9 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
     // h = act_a tanh(acc) + act_b; the tanh form keeps the sigmoid's instruction
     // pattern (one packed fma after the tanh)
     constexpr uint32_t act_a = tanh_act ? BF2_ONE : BF2_HALF, act_b = tanh_act ? 0u : BF2_HALF;
-    auto bar_count = [&](int i) -> uint32_t {   // in address order, from Z1F on
-        const int k = i - 2 * NSTAGE;
-        if (k == 5 || k == 6 || k == 9 || k == 10) return NGRP_T;   // DF, EPI
-        if (k == 8 || k == 11) return NEPI_T;                       // W, EPIA
+    auto bar_count = [&](int i) -> uint32_t {
+        if ((i >= I_DF && i < I_DF + NDF) || i == I_EPI || i == I_EPI + 1) return NGRP_T;
+        if (i == I_W || i == I_EPIA) return NEPI_T;
         return 1;
     };
 
@@ -220,7 +233,7 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
             const int nks = D / 16 + 1;   // K = D + 1 in steps of 16
             const uint64_t xd0 = sdesc(sb + SM_X, 16, 1024, 2);
             const uint64_t wd0 = sdesc(sb + SM_W1, 16, 1024, 2);
-            int t = 0, e = 0, s = 0, sph = 0, buf = 0, bph = 1;   // bph: parity of GD's previous phase
+            int t = 0, e = 0, s = 0, sph = 0, buf = 0, bph = 1;   // bph: parity of GD's phase before
             bool go = true;
             for (int it = 0; it < total && go; ++it) {
                 go = __all_sync(0xffffffffu, mbar_wait(BAR_FULL + 8 * s, sph, abort));
@@ -245,10 +258,10 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
                             for (int ks = 0; ks < 4; ++ks)
                                 if (ks < nks) mma_bf16(dt, wd + ks * 2, xd + ks * 2, id_fwd, ks > 0 ? 1u : 0u);
                         }
-                        mma_commit(BAR_Z1F + 8 * g);
+                        mma_commit(BAR_Z1F + 8 * (NZ1 * g + buf));
                     }
                     __syncwarp();
-                    if (++buf == 3) { buf = 0; bph ^= 1; }
+                    if (++buf == NZ1) { buf = 0; bph ^= 1; }
                 }
                 if (++s == NSTAGE) { s = 0; sph ^= 1; }
                 if (++t == T) { t = 0; ++e; }
@@ -274,14 +287,14 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
                 };
                 bool ok = true;
                 while (ok && issued < NSTAGE && issued < total) ok = load();
-                int t = 0, s = 0, sph = 0, buf = 0;
+                int t = 0, s = 0, sph = 0, buf = 0, bph = 0;
                 for (int it = 0; it < total && ok; ++it) {
                     // the stage of tile it - 1 is free once its MMAs are done
                     if (it > 0 && issued < total && !load()) { ok = false; break; }
                     if (!mbar_wait(BAR_FULL + 8 * s, sph, abort)) { ok = false; break; }
                     for (int g = 0; g < 2; ++g) {
                         // [gW1 | gb1] / w2 += d1^T [X | 1]
-                        if (!mbar_wait(BAR_DF + 8 * g, it & 1, abort)) { ok = false; break; }
+                        if (!mbar_wait(BAR_DF + 8 * buf, bph, abort)) { ok = false; break; }
                         tc_fence_after();
                         const uint64_t xd = xd0 + (uint32_t)(s * (16384 >> 4) + g * (8192 >> 4));
                         for (int b = 0; b < NB; ++b) {
@@ -292,7 +305,7 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
                                             (t > 0 || g > 0 || kk > 0) ? 1u : 0u);
                         }
                         mma_commit(BAR_GD + 8 * buf);
-                        if (++buf == 3) buf = 0;
+                        if (++buf == NZ1) { buf = 0; bph ^= 1; }
                     }
                     if (!ok) break;
                     mma_commit(BAR_EMPTY + 8 * s);
@@ -319,7 +332,7 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
             float *zx = (float *)(sm + SM_ZX) + 512 * g;                       // [2][4 quarters][64 rows]
             uint32_t *dsm = (uint32_t *)(sm + SM_D2) + 16 * (warp - 2);        // 32 rows' d2 in bf16 pairs
             float b2 = P[HD + 2 * H];
-            int it = 0, buf = g, epi_use = 0;
+            int it = 0, buf = g, bph = 0, epi_use = 0;   // bph: parity of this group's use of a buffer
             bool ok = true;
             // Barrier of all epilogue threads with a bounded wait (an mbarrier, so
             // that a block that aborts cannot leave it hanging).
@@ -342,7 +355,7 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
                     const float yv = y_next;
                     if (row + TR < n) y_next = nd.y[row + TR];
                     const uint32_t zc = lane_base + TM_Z1 + 128 * buf;
-                    if (!mbar_wait(BAR_Z1F + 8 * g, it & 1, abort)) { ok = false; break; }
+                    if (!mbar_wait(BAR_Z1F + 8 * (NZ1 * g + buf), bph, abort)) { ok = false; break; }
                     tc_fence_after();
                     // pass 1: h in bf16 pairs of rows, and the warp's share of z2 = h w2
                     // (FP32), 16 rows at a time
@@ -417,8 +430,9 @@ __global__ void __launch_bounds__(NT, 1) k_tc_batched(TcArgs a) {
                         tmem_st16(zc + 64 * b + 16 * rh, d1);
                     }
                     tc_fence_before();
-                    mbar_arrive(BAR_DF + 8 * g);
-                    buf = buf == 0 ? 2 : buf - 1;   // two subtiles on, modulo 3
+                    mbar_arrive(BAR_DF + 8 * buf);
+                    buf = buf == 0 ? NZ1 - 1 : buf - 1;   // two half tiles on, modulo 3
+                    if (buf == g) bph ^= 1;               // the group has used all three
                 }
                 if (!ok) break;
                 // ---- end of epoch: reductions and the update

@@ -240,3 +240,47 @@ def test_config_1024_nets_200_epochs_against_stored_oracle_runs():
         w0 = WL.kept_params(*W[t], WL.C4_KEEP_EVERY)
         got = WL.kept_params(pg.W1, pg.b1, pg.w2, pg.b2, WL.C4_KEEP_EVERY)
         assert rel_err_norm(got - w0, np.asarray(g["kept_params"]) - w0) <= BF16_GRAD_TOL, t
+
+
+@pytest.mark.parametrize("D_real,D_pad", [(5, 8), (13, 16), (50, 56)])
+@pytest.mark.parametrize("H", [128, 256])
+def test_several_epochs_at_the_edges_of_tiles(D_real, D_pad, H):
+    """Six epochs of nets with one to five tiles of 128 rows, the last with 1 to
+    128 rows (either or both of its halves of 64): more half tiles than Z1
+    buffers and stages, the shortest products (D = 8) among them.  The weights'
+    movement within the bf16 gradient bar of every epoch's largest gradient; the
+    gradient's own drift with the weights (lr x curvature, below a tenth) adds a
+    tenth."""
+    epochs, lr = 6, lr32()
+    nets = []
+    for i, n in enumerate((1, 64, 65, 128, 129, 192, 193, 257, 385, 600)):
+        X = I.bf16_round(I.features(5300 + 10 * D_pad + i, n, D_real, D_pad))
+        y = (X[:, 0] + X[:, 1] > 0).astype(np.float32)
+        nets.append((X, y, I.init_weights(5400 + 10 * D_pad + i, D_real, H, D_pad)))
+    keep, descs, params, losses = [], [], [], []
+    import torch
+    for X, y, W in nets:
+        Xd, yd = dev(I.bf16_bits(X).view(np.int16)), dev(y)
+        P = dev(flat(W).astype(np.float32))
+        L = torch.zeros(epochs, dtype=torch.float64, device="cuda")
+        keep += [Xd, yd]
+        params.append(P)
+        losses.append(L)
+        descs.append(B.mlp_net_desc(H, X.shape[0], Xd.data_ptr(), yd.data_ptr(), P.data_ptr(), L.data_ptr()))
+    b = B.mlp_batch_create(B.MLP_BF16, B.MLP_ACT_SIGMOID, D_pad, descs, lr, 1)
+    try:
+        B.mlp_batch_run(b, epochs, stream())
+        assert B.mlp_batch_check(b, stream()) == B.MLP_OK, B.mlp_last_error()
+    finally:
+        B.mlp_batch_destroy(b)
+    for (X, y, W), P, L in zip(nets, params, losses):
+        p, bound = flat(W), 0.0
+        for _ in range(epochs):
+            HD = H * D_pad
+            g = oracle.mse_gradients(X, y, Params(p[:HD].reshape(H, D_pad), p[HD:HD + H], p[HD + H:HD + 2 * H], p[-1]))
+            g = np.concatenate([np.ravel(a) for a in g[:4]])
+            p = p - lr * g
+            bound += lr * np.max(np.abs(g))
+        assert np.max(np.abs(host(P) - p)) <= 1.1 * BF16_GRAD_TOL * bound, len(y)
+        _, lh, _ = oracle.train(X, y, Params(*W), lr, epochs)
+        assert rel_err_elem(host(L), lh) <= 2e-2, len(y)
