@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
         int64_t lo[2], hi[2];   // this block's rows of a full step [0] and of the last, ragged one [1]
         float c[2];             // and the scale of their output deltas
         double sse;             // one block: squared error of the epoch so far
-        long long fix;          // several: the same as the sum of the steps' fixed-point values
+        double sum;             // several: the same
         int64_t step;           // one block: of the epoch, the next step to finish
         int epoch;              //   and its epoch
     } sv;
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
     }
     if (tid == 4) {
         sv.sse = 0.0;
-        sv.fix = 0;
+        sv.sum = 0.0;
         sv.step = 0;
         sv.epoch = 0;
     }
@@ -357,11 +357,13 @@ __global__ void __launch_bounds__(FNT, 1) k_fused_train(FArgs a) {
                 }
                 __syncthreads();
                 if (tid == 0) {
-                    sv.fix += s_sse;   // at most n 2^32 and a rounding a block and step: exact
+                    // FP64 over the steps: only a step's fixed-point sum is checked against its
+                    // range, an epoch's could leave it (labels of some hundreds)
+                    sv.sum += (double)s_sse * (1.0 / 4294967296.0);
                     if (epoch_end) {
                         const double Cl = a.loss_mean ? 1.0 / (double)a.n : 1.0;
-                        const double L = 0.5 * ((double)sv.fix * (1.0 / 4294967296.0)) * Cl;
-                        sv.fix = 0;
+                        const double L = 0.5 * sv.sum * Cl;
+                        sv.sum = 0.0;
                         if (a.loss_hist) a.loss_hist[e] = L;
                         if (!isfinite(L)) atomicOr(a.status, ST_NONFINITE);
                         if (want_gn) {

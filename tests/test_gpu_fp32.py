@@ -436,3 +436,21 @@ def test_train_path_names_the_kernel_a_shape_takes():
     for (D, H, prec), want in cases:
         with Net(D, H, prec=prec) as net:
             assert B.mlp_train_path(net.h, 1000, 0) == want, (D, H, prec)
+
+
+def test_epoch_loss_beyond_a_steps_fixed_point_range():
+    """Labels near 400 in mini-batches over several blocks: every step's squared
+    error (1.6e8) is within the fixed-point range, the epoch's (3.2e9) beyond 2^31.
+    A squared error carries 2^-23 of rounding, a lane's sum of at most 64 of them
+    4e-6: 1e-5."""
+    t = torch()
+    n = 20011
+    X, _, W = problem(88, n, 33, 100)
+    y = (400.0 + np.random.default_rng(88).normal(size=n)).astype(np.float32)
+    lh = t.zeros(3, dtype=t.float64, device="cuda")
+    with Net(33, 100, lr=1e-5) as net:
+        net.set(W)
+        B.mlp_train_epochs(net.h, dev(X), dev(y), n, 3, 1000, lh, None, stream())
+        assert net.check() == B.MLP_OK
+    _, ref, _ = oracle.train(X, y, Params(*W), lr32(1e-5), 3, minibatch=1000)
+    np.testing.assert_allclose(host(lh), ref, rtol=1e-5)
