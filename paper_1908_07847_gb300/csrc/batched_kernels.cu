@@ -18,12 +18,13 @@ constexpr int BCAP = 256;        // rows staged in shared memory at a time
 
 constexpr int RING = 32;         // epochs whose losses are finished together
 
-// RB1, RBN: rows a lane keeps in flight for H <= 32 and above.
+// RB1, RBN: rows a lane keeps in flight for H <= 32 and above, whole deals of one
+// and RE_RB rows in both forms: a net's bits do not depend on the plan's size.
 template <int DP, int WU, int ACT, int RB1, int RBN, bool ONE>
 __device__ __forceinline__ void net_body(const BatchNet &nd, int D, int epochs, float lr, int loss_mean,
                                          int *status, float *Xs, float *ys, float *Wm, float *part,
                                          float *zx, double (*s_sse)[RE_NW], double *s_gn) {
-    using Eng = RowEngine<DP, WU, ACT, RB1, RBN>;
+    using Eng = RowEngine<DP, WU, ACT, RB1, RBN, 1, RE_RB>;
     Eng eng;
     eng.setup(nd.H, D);
     constexpr int NG = Eng::NG;

@@ -34,12 +34,16 @@ __host__ __device__ inline int re_groups(int H) { return RE_NW / re_wu(H); }
 
 // Rows in flight per lane: RB1 when H <= 32 (segments of a warp already take
 // separate rows there), RBN otherwise; a kernel with the register file to
-// itself can afford more than the defaults.
-template <int DP, int WU, int ACT, int RB1 = 2, int RBN = RE_RB>
+// itself can afford more than the defaults.  Rows are dealt to the row groups
+// GR1 (GRN) at a time: two forms of a kernel that agree in these add every row
+// to the same sums in the same order, whatever they keep in flight.
+template <int DP, int WU, int ACT, int RB1 = 2, int RBN = RE_RB, int GR1 = RB1, int GRN = RBN>
 struct RowEngine {
     static_assert(RB1 <= RE_RB_MAX && RBN <= RE_RB_MAX, "z2 exchange space");
+    static_assert(RB1 % GR1 == 0 && RBN % GRN == 0, "whole deals in flight");
     static constexpr int NG = RE_NW / WU;
     static constexpr int RB = (WU == 1) ? RB1 : RBN;
+    static constexpr int GR = (WU == 1) ? GR1 : GRN;
     // Per-lane state: the neuron's weights and gradient sums.
     float w[DP];
     float acc[DP];
@@ -79,100 +83,113 @@ struct RowEngine {
         sse = 0.0;
     }
 
+    // One turn of R rows a lane (R = RB, or GR), the slot's first at base + slot.
+    // Row t of a slot's batch is base + t * nslots + slot (every GR rows a deal
+    // further): neighbouring segments read neighbouring rows, whose float4 words
+    // fall in distinct shared-memory banks (row stride DP = 4 mod 32 words or a
+    // multiple of 8).
+    template <int R>
+    __device__ __forceinline__ void turn(const float *Xs, const float *ys, int base, int cn, float c, float *zx,
+                                         float &sse_f) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int grp = warp / WU, wu = warp % WU;
+        const int nslots = 32 / S, slot = lane / S, deal = nslots * GR;
+        int xo[R], rr[R];
+        bool valid[R];
+#pragma unroll
+        for (int t = 0; t < R; ++t) {
+            rr[t] = base + (t / GR) * NG * deal + (t % GR) * nslots + slot;
+            valid[t] = rr[t] < cn;
+            xo[t] = (valid[t] ? rr[t] : 0) * DP;
+        }
+        float z[R];
+#pragma unroll
+        for (int t = 0; t < R; ++t) z[t] = b1r;
+#pragma unroll
+        for (int q = 0; q < DP / 4; ++q) {
+#pragma unroll
+            for (int t = 0; t < R; ++t) {
+                const float4 xv = *reinterpret_cast<const float4 *>(Xs + xo[t] + 4 * q);
+                z[t] = fmaf(xv.x, w[4 * q + 0], z[t]);
+                z[t] = fmaf(xv.y, w[4 * q + 1], z[t]);
+                z[t] = fmaf(xv.z, w[4 * q + 2], z[t]);
+                z[t] = fmaf(xv.w, w[4 * q + 3], z[t]);
+            }
+        }
+        // Re-read the rows from shared memory in the backward pass instead of
+        // keeping R x DP values live in registers.
+        asm volatile("" ::: "memory");
+        float hv[R], zp[R];
+#pragma unroll
+        for (int t = 0; t < R; ++t) {
+            hv[t] = Act<ACT>::f(z[t]);
+            zp[t] = hv[t] * w2r;
+        }
+        // Butterfly over the segment, level by level so that the R rows'
+        // shuffles overlap.
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            if (WU > 1 || off < S) {
+#pragma unroll
+                for (int t = 0; t < R; ++t) zp[t] += __shfl_xor_sync(0xffffffffu, zp[t], off);
+            }
+        }
+        if (WU > 1) {
+            // (the buffers keep their places for every R)
+            float *zg = zx + (par * NG + grp) * (WU * RB);
+            if (lane == 0) {
+#pragma unroll
+                for (int t = 0; t < R; ++t) zg[wu * RB + t] = zp[t];
+            }
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(WU * 32) : "memory");
+#pragma unroll
+            for (int t = 0; t < R; ++t) {
+                float v = zg[t];
+#pragma unroll
+                for (int q = 1; q < WU; ++q) v += zg[q * RB + t];
+                zp[t] = v;
+            }
+            par ^= 1;
+        }
+#pragma unroll
+        for (int t = 0; t < R; ++t) {
+            const float o = sigmoid_out(zp[t] + b2);
+            const float err = o - ys[valid[t] ? rr[t] : 0];
+            const float d2 = valid[t] ? c * err * o * (1.0f - o) : 0.f;
+            if (valid[t]) sse_f = fmaf(err, err, sse_f);
+            gb2a += d2;
+            gw2a = fmaf(d2, hv[t], gw2a);
+            const float d1 = d2 * w2r * Act<ACT>::df(hv[t]);
+            gb1a += d1;
+            hv[t] = d1;
+        }
+#pragma unroll
+        for (int q = 0; q < DP / 4; ++q) {
+#pragma unroll
+            for (int t = 0; t < R; ++t) {
+                const float4 xv = *reinterpret_cast<const float4 *>(Xs + xo[t] + 4 * q);
+                acc[4 * q + 0] = fmaf(hv[t], xv.x, acc[4 * q + 0]);
+                acc[4 * q + 1] = fmaf(hv[t], xv.y, acc[4 * q + 1]);
+                acc[4 * q + 2] = fmaf(hv[t], xv.z, acc[4 * q + 2]);
+                acc[4 * q + 3] = fmaf(hv[t], xv.w, acc[4 * q + 3]);
+            }
+        }
+    }
+
     // Rows 0..cn-1 of the staged chunk Xs (DP floats per row, zero padded) with
     // labels ys; c scales the output delta (1/m or 1).
     __device__ __forceinline__ void rows(const float *Xs, const float *ys, int cn, float c, float *zx) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        const int grp = warp / WU, wu = warp % WU;
-        const int slot = lane / S;
-        const int RPI = (32 / S) * RB;
         // Squared errors of this call are summed in FP32 per lane and folded
         // into the FP64 sum once (FP64 arithmetic is slow on this part).
         float sse_f = 0.f;
-        // Row t of a slot's batch is base + t * nslots + slot: neighbouring
-        // segments read neighbouring rows, whose float4 words fall in distinct
-        // shared-memory banks (row stride DP = 4 mod 32 words or a multiple of 8).
-        const int nslots = 32 / S;
-        for (int base = grp * RPI; base < cn; base += NG * RPI) {
-            int xo[RB], rr[RB];
-            bool valid[RB];
-#pragma unroll
-            for (int t = 0; t < RB; ++t) {
-                rr[t] = base + t * nslots + slot;
-                valid[t] = rr[t] < cn;
-                xo[t] = (valid[t] ? rr[t] : 0) * DP;
-            }
-            float z[RB];
-#pragma unroll
-            for (int t = 0; t < RB; ++t) z[t] = b1r;
-#pragma unroll
-            for (int q = 0; q < DP / 4; ++q) {
-#pragma unroll
-                for (int t = 0; t < RB; ++t) {
-                    const float4 xv = *reinterpret_cast<const float4 *>(Xs + xo[t] + 4 * q);
-                    z[t] = fmaf(xv.x, w[4 * q + 0], z[t]);
-                    z[t] = fmaf(xv.y, w[4 * q + 1], z[t]);
-                    z[t] = fmaf(xv.z, w[4 * q + 2], z[t]);
-                    z[t] = fmaf(xv.w, w[4 * q + 3], z[t]);
-                }
-            }
-            // Re-read the rows from shared memory in the backward pass instead of
-            // keeping RB x DP values live in registers.
-            asm volatile("" ::: "memory");
-            float hv[RB], zp[RB];
-#pragma unroll
-            for (int t = 0; t < RB; ++t) {
-                hv[t] = Act<ACT>::f(z[t]);
-                zp[t] = hv[t] * w2r;
-            }
-            // Butterfly over the segment, level by level so that the RB rows'
-            // shuffles overlap.
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                if (WU > 1 || off < S) {
-#pragma unroll
-                    for (int t = 0; t < RB; ++t) zp[t] += __shfl_xor_sync(0xffffffffu, zp[t], off);
-                }
-            }
-            if (WU > 1) {
-                float *zg = zx + (par * NG + grp) * (WU * RB);
-                if (lane == 0) {
-#pragma unroll
-                    for (int t = 0; t < RB; ++t) zg[wu * RB + t] = zp[t];
-                }
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(WU * 32) : "memory");
-#pragma unroll
-                for (int t = 0; t < RB; ++t) {
-                    float v = zg[t];
-#pragma unroll
-                    for (int q = 1; q < WU; ++q) v += zg[q * RB + t];
-                    zp[t] = v;
-                }
-                par ^= 1;
-            }
-#pragma unroll
-            for (int t = 0; t < RB; ++t) {
-                const float o = sigmoid_out(zp[t] + b2);
-                const float err = o - ys[valid[t] ? rr[t] : 0];
-                const float d2 = valid[t] ? c * err * o * (1.0f - o) : 0.f;
-                if (valid[t]) sse_f = fmaf(err, err, sse_f);
-                gb2a += d2;
-                gw2a = fmaf(d2, hv[t], gw2a);
-                const float d1 = d2 * w2r * Act<ACT>::df(hv[t]);
-                gb1a += d1;
-                hv[t] = d1;
-            }
-#pragma unroll
-            for (int q = 0; q < DP / 4; ++q) {
-#pragma unroll
-                for (int t = 0; t < RB; ++t) {
-                    const float4 xv = *reinterpret_cast<const float4 *>(Xs + xo[t] + 4 * q);
-                    acc[4 * q + 0] = fmaf(hv[t], xv.x, acc[4 * q + 0]);
-                    acc[4 * q + 1] = fmaf(hv[t], xv.y, acc[4 * q + 1]);
-                    acc[4 * q + 2] = fmaf(hv[t], xv.z, acc[4 * q + 2]);
-                    acc[4 * q + 3] = fmaf(hv[t], xv.w, acc[4 * q + 3]);
-                }
-            }
+        const int grp = (threadIdx.x >> 5) / WU, deal = 32 / S * GR;
+        for (int base = grp * deal; base < cn; base += NG * (32 / S) * RB) {
+            // A last turn of one deal takes no more rows than it has (100 nets of 4 to
+            // 128 units, 50 to 120 rows, one block an SM: 9877 us without, 9011 so).  With
+            // a warp a group a turn's few rows cost nothing (two nets of 45 rows: 2323
+            // us, 2378 with the second form of the loop).
+            if (WU > 1 && RB > GR && base + NG * deal >= cn) turn<GR>(Xs, ys, base, cn, c, zx, sse_f);
+            else turn<RB>(Xs, ys, base, cn, c, zx, sse_f);
         }
         sse += (double)sse_f;
     }

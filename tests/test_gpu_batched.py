@@ -312,3 +312,24 @@ def test_shape_validation_and_autotuner(tmp_path, monkeypatch):
             assert e.value.status == B.MLP_EINVAL
     finally:
         B.mlp_batch_destroy(b)
+
+
+@pytest.mark.parametrize("D,H_lo,H_hi", [(33, 4, 128), (8, 1, 32), (16, 33, 64), (60, 4, 128)])
+def test_net_result_does_not_depend_on_the_plans_size(D, H_lo, H_hi):
+    """More nets than SMs in one plan (two blocks an SM where they fit) and the
+    same nets in two smaller plans (one block an SM, more rows in flight), as two
+    ranks would train their shares: the same bits.  Rows from one to beyond the
+    256 that a block stages at a time."""
+    t = torch()
+    N = t.cuda.get_device_properties(0).multi_processor_count + 8
+    rng = np.random.default_rng(D)
+    nets = []
+    for i in range(N):
+        n, H = int(rng.integers(1, 300)), int(rng.integers(H_lo, H_hi + 1))
+        X = rng.normal(size=(n, D)).astype(np.float32)
+        nets.append((X, (X[:, 0] > 0).astype(np.float32), I.init_weights(900 + i, D, H)))
+    whole, lw = run_batch(nets, 12, D=D)
+    for part in (range(0, N // 2), range(N // 2, N)):
+        got, lg = run_batch([nets[i] for i in part], 12, D=D)
+        for k, i in enumerate(part):
+            assert np.array_equal(got[k], whole[i]) and np.array_equal(lg[k], lw[i]), i
