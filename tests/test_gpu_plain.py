@@ -121,3 +121,56 @@ def test_tensor_core_forward_of_values_outside_the_parts_range(where):
     assert np.isnan(got[600]) and np.isnan(ref[600])
     ok = np.arange(n) != 600
     assert rel_err_elem(got[ok], ref[ok]) <= FWD_TOL
+
+
+@pytest.mark.parametrize("prec,D,H,n", [("fp32", 33, 2000, 9000), ("fp32", 12, 1940, 9000), ("fp32", 64, 2048, 8100),
+                                        ("bf16", 48, 2000, 14000), ("bf16", 19, 2048, 13000)])
+def test_tensor_core_forward_between_plain_tiles(prec, D, H, n):
+    """Blocks that walk over several tiles, some outside the parts' range (every
+    third tile, by one row) and some not: units go back and forth between their
+    parts and their plain form, with remainders of inputs, rows and units, and
+    once with a block of units that never has parts (a weight of 1e-33)."""
+    import torch
+    from paper_1908_07847_gb300 import inputs as I
+    X, _, W = problem(7500 + D, n, D, H)
+    for r, v in zip(range(5, n, 384), [np.inf, -2.0 ** 62, 3e38, 1e-33] * n):
+        X[r, r % D] = v
+    if prec == "bf16":
+        X = I.bf16_round(X)
+    W[0][H - 1, 1] = 1e-33
+    with Net(D, H, prec=B.MLP_BF16 if prec == "bf16" else B.MLP_FP32) as net:
+        net.set(W)
+        o = torch.zeros(n, device="cuda")
+        B.mlp_forward(net.h, dev(X).to(torch.bfloat16 if prec == "bf16" else torch.float32), n, o, stream())
+        got = host(o)
+    with np.errstate(all="ignore"):
+        _, ref = oracle.forward(X, Params(*W))
+    assert np.all(np.isfinite(ref)) and rel_err_elem(got, ref) <= FWD_TOL
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_plain_tiles_of_the_tensor_core_forward_are_not_slow(prec):
+    """A fit that diverged, or one tiny or infinite weight a block of units, sends
+    every tile through multiply-adds: some five times the clean call's time, 20 to 90
+    times when each multiply-add loaded its operands.  Bound: 10."""
+    import torch
+    n, D, H = 100003, 48, 1024
+    X = torch.randn((n, D), device="cuda").to(torch.bfloat16 if prec == "bf16" else torch.float32)
+    o = torch.zeros(n, device="cuda")
+    times = []
+    for bad in (False, True):
+        _, _, W = problem(7600, 16, D, H)
+        if bad:
+            W[0][::128, 3] = 1e-33
+        with Net(D, H, prec=B.MLP_BF16 if prec == "bf16" else B.MLP_FP32) as net:
+            net.set(W)
+            t = []
+            for _ in range(6):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                B.mlp_forward(net.h, X, n, o, stream())
+                b.record()
+                torch.cuda.synchronize()
+                t.append(a.elapsed_time(b))
+        times.append(min(t[1:]))
+    assert times[1] <= 10 * times[0], times
