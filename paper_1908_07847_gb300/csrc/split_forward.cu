@@ -7,9 +7,15 @@
 // which the three below 2^-24 x w are left out; for bf16 rows only w is cut, and
 // nothing is left out.  tcgen05.mma adds them in FP32, but rounds towards zero at
 // every accumulation, so the small products go first: three (D <= 48) or four
-// accumulations meet a sum of full size.  Measured against 64 bits on N(0, 1)
-// values, 2-norm relative: K = 48 6.6e-8 (chain of FP32 multiply-adds 1.26e-7),
-// K = 64 7.5e-8 (1.46e-7), bf16 rows K = 48 5.2e-8 (big products first: 5.6e-7).
+// accumulations meet a sum of full size.  For FP32 rows the steps' large products
+// are shared between two accumulators, added rounded to nearest, so at most two do;
+// bf16 rows keep one (two take the tensor memory of the third block an SM: the
+// 200003 rows below 368 -> 412 us).  Measured against 64 bits, root mean square
+// error / sum |x w| (chains of FP32 multiply-adds in brackets), D = 16, 33, 48, 64:
+//   x N(0, 1), w U(-1, 1)   1.7 1.5 1.1 1.0e-8 (2.6), bf16 rows 1.7 - 1.4 1.3e-8
+//   both U(0, 1)            5.1 6.0 5.0 5.7e-8 (6.2 8.4 10 11), bf16 5.1 - 6.9 8.3e-8
+//   x exp(3 N(0, 1)), w U(0, 1), where mostly one term counts and the bias adds up:
+//                           6.1 11 10 12e-8 (6.8 9.4 11 13), bf16 6.1 - 16 23e-8
 //
 // One block takes 128 units (W1's parts stay in shared memory) and walks over
 // tiles of 128 rows: M = 128 rows, N = 128 units, K = 16 at a time, 64 clocks an
@@ -44,6 +50,7 @@ constexpr int SU = 128;          // units of a block
 constexpr uint32_t PART = 16384; // one part of a tile: 128 rows of 128 bytes (64 inputs), 128-byte swizzle
 
 template <typename TX> constexpr int x_parts = std::is_same<TX, float>::value ? 3 : 1;
+template <typename TX> constexpr int tm_cols = x_parts<TX> == 3 ? 2 * SU : SU;   // tensor memory: accumulators of SU columns
 constexpr int WIN = 2048;        // a block's tiles between two turns of its plain ones
 template <typename TX> constexpr uint32_t split_smem = (x_parts<TX> + 3) * PART + 2 * SU * 4 + 64 + WIN / 8 + 1024;
 
@@ -172,7 +179,8 @@ k_fwd_split(int D, int H, int64_t n, const TX *__restrict__ X, const float *__re
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(s32(tmem_slot)));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(tmem_slot)),
+                     "n"(tm_cols<TX>));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     // this block's units in parts; whether one cannot be
@@ -262,11 +270,15 @@ k_fwd_split(int D, int H, int64_t n, const TX *__restrict__ X, const float *__re
                     constexpr int XP[6] = {2, 0, 1, 1, 0, 0}, WP[6] = {0, 2, 1, 0, 1, 0};
 #pragma unroll
                     for (int c = 0; c < (NX == 3 ? 6 : 3); ++c) {
+                        // of the large products, the steps from k2 on go to the second accumulator
+                        const int k2 = NX == 3 && c == 5 ? (nks + 1) >> 1 : 4;
                         const uint64_t xa = xd + (NX == 3 ? XP[c] : 0) * (PART >> 4);
                         const uint64_t wb = wd + (NX == 3 ? WP[c] : 2 - c) * (PART >> 4);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            if (ks < nks) mma_bf16(tmem, xa + 2 * ks, wb + 2 * ks, id, (c > 0 || ks > 0) ? 1u : 0u);
+                            if (ks < nks)
+                                mma_bf16(ks < k2 ? tmem : tmem + SU, xa + 2 * ks, wb + 2 * ks, id,
+                                         ks != k2 && (c > 0 || ks > 0) ? 1u : 0u);
                     }
                     mma_commit(bar);
                 }
@@ -286,6 +298,15 @@ k_fwd_split(int D, int H, int64_t n, const TX *__restrict__ X, const float *__re
             for (int c = 0; c < 64; c += 32) {
                 float z[32];
                 tmem_ld32(lane_base + c, z);
+                if (NX == 3 && nks > 1) {
+#pragma unroll
+                    for (int v = 0; v < 32; v += 16) {
+                        float z2[16];
+                        tmem_ld16(lane_base + SU + c + v, z2);
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) z[v + u] += z2[u];
+                    }
+                }
 #pragma unroll
                 for (int u = 0; u < 32; u += 4) {
                     const float4 bv = *(const float4 *)(b1s + c0 + c + u), wv = *(const float4 *)(w2s + c0 + c + u);
@@ -341,7 +362,7 @@ k_fwd_split(int D, int H, int64_t n, const TX *__restrict__ X, const float *__re
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(tm_cols<TX>));
 }
 
 template <typename TX, int ACT>
