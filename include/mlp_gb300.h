@@ -99,7 +99,12 @@ mlp_status mlp_get_weights(mlp_t net, void *W1_host, void *b1_host,
  * mlp_destroy). */
 mlp_status mlp_weights_device(mlp_t net, void **params_dev);
 
-/* Forward pass (Sec. 2.2, Eq. 1) with the handle's weights: writes o [n]. */
+/* Forward pass (Sec. 2.2, Eq. 1) with the handle's weights: writes o [n].  The
+ * same call gives the same bits.  For FP32 and bf16 rows with 12 <= D <= 64 and
+ * H > 64 the kernel, and so the order of a row's sums, follows n (large calls run
+ * on the tensor cores), and whether hidden activations are stored: scores of a
+ * table taken in pieces agree with those taken at once within the FP32 bar, not
+ * bit for bit. */
 mlp_status mlp_forward(mlp_t net, const void *X, int64_t n, void *o, void *stream);
 
 /* Squared-error gradients at the handle's weights (Sec. 2.2 backpropagation):
@@ -184,7 +189,9 @@ mlp_status mlp_train_host(mlp_t net, const void *X_host, const void *y_host,
                           int64_t n, int32_t epochs, int64_t minibatch,
                           double *loss_hist_host, void *stream);
 
-/* Classification (Sec. 2.2): labels[i] = 1 iff o_i >= 0.5, else 0. */
+/* Classification (Sec. 2.2): labels[i] = 1 iff o_i >= 0.5, else 0, with o as
+ * mlp_forward gives it for the same n (an o within rounding of 0.5 may fall on
+ * the other side in a call of another n). */
 mlp_status mlp_predict(mlp_t net, const void *X, int64_t n, int8_t *labels, void *stream);
 
 /* Synchronise `stream`, then return and clear the handle's device status:

@@ -194,3 +194,31 @@ def test_tensor_core_forward_of_rows_with_one_dominant_term(D, H, n):
     B.mlp_forward_w(B.MLP_FP32, B.MLP_ACT_TANH, D, H, n, dev(X), *[dev(w) for w in W], hd, o, ws, nb, stream())
     ref = np.tanh(X.astype(np.float64) @ W[0].astype(np.float64).T)
     assert abs(np.mean(host(hd) / ref - 1)) <= 1.3e-7
+
+
+@pytest.mark.parametrize("prec,D,H", [("fp32", 33, 512), ("bf16", 48, 2048)])
+def test_scores_in_pieces_agree_with_scores_at_once(prec, D, H):
+    """A table scored at once (tensor cores) and 500 rows at a time (multiply-add
+    chains): each within the forward bar of the oracle, so within twice of each
+    other; labels differ only where o is that near 0.5.  The same call again gives
+    the same bits."""
+    import torch
+    n = 20000
+    X, _, W = problem(7700, n, D, H)
+    Xd = dev(X).to(torch.bfloat16 if prec == "bf16" else torch.float32)
+    whole, again, pieces = (torch.zeros(n, device="cuda") for _ in range(3))
+    lab, labp = (torch.zeros(n, dtype=torch.int8, device="cuda") for _ in range(2))
+    with Net(D, H, prec=B.MLP_BF16 if prec == "bf16" else B.MLP_FP32) as net:
+        net.set(W)
+        B.mlp_forward(net.h, Xd, n, whole, stream())
+        B.mlp_forward(net.h, Xd, n, again, stream())
+        B.mlp_predict(net.h, Xd, n, lab, stream())
+        for i in range(0, n, 500):
+            B.mlp_forward(net.h, Xd[i:i + 500], 500, pieces[i:i + 500], stream())
+            B.mlp_predict(net.h, Xd[i:i + 500], 500, labp[i:i + 500], stream())
+        torch.cuda.synchronize()
+    assert torch.equal(whole, again)
+    assert rel_err_elem(host(pieces), host(whole)) <= 2 * FWD_TOL
+    o = host(whole).astype(np.float64)
+    assert np.array_equal(host(lab), (o >= 0.5).astype(np.int8))
+    assert np.all(np.abs(o - 0.5)[host(lab) != host(labp)] <= FWD_TOL)
