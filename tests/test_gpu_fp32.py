@@ -454,3 +454,26 @@ def test_epoch_loss_beyond_a_steps_fixed_point_range():
         assert net.check() == B.MLP_OK
     _, ref, _ = oracle.train(X, y, Params(*W), lr32(1e-5), 3, minibatch=1000)
     np.testing.assert_allclose(host(lh), ref, rtol=1e-5)
+
+
+@pytest.mark.parametrize("n,mb,rows", [(1003, 500, None), (1003, 500, 64), (2433, 2432, None), (5000, 2433, None),
+                                       (1237, 600, 150), (66, 33, None), (65, 33, 17)])
+def test_minibatches_loaded_ahead_with_ragged_last_steps(n, mb, rows):
+    """Mini-batches over several blocks: rows loaded a step ahead (at most 64 a
+    block) or in chunks (150), a last step of fewer rows than blocks or of one
+    row, the default rows a block on both sides of its rule; weights, loss and
+    gradient-norm histories against the oracle."""
+    D, H, epochs = 33, 40, 6
+    X, y, W = problem(1800 + n, n, D, H)
+    t = torch()
+    lh, gh = (t.zeros(epochs, dtype=t.float64, device="cuda") for _ in range(2))
+    with Net(D, H) as net:
+        net.set(W)
+        if rows:
+            B.mlp_set_rows_per_block(net.h, rows)
+        B.mlp_train_epochs(net.h, dev(X), dev(y), n, epochs, mb, lh, gh, stream())
+        assert net.check() == B.MLP_OK, B.mlp_last_error()
+        q, lh_ref, gh_ref = oracle.train(X, y, Params(*W), lr32(), epochs, minibatch=mb)
+        assert rel_err_norm(net.flat(), q.flat()) <= W_TOL
+        assert rel_err_elem(host(lh), lh_ref) <= 1e-5
+        assert rel_err_elem(host(gh), gh_ref) <= 1e-4
