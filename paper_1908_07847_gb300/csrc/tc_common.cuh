@@ -205,9 +205,6 @@ __device__ __forceinline__ void fma_rows(uint32_t a, uint32_t b, float &acc0, fl
         : "+f"(acc0), "+f"(acc1)
         : "r"(a), "r"(b));
 }
-// sigmoid of a pair given half its argument: 1/2 + tanh(x/2)/2.
-__device__ __forceinline__ uint32_t sigmoid_half_bf2(uint32_t xhalf) { return hfma2(tanh_bf2(xhalf), BF2_HALF, BF2_HALF); }
-
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t *>(&v);
