@@ -106,8 +106,9 @@ __device__ __forceinline__ void add_group(double &acc, const float (&v)[N], cons
 }
 
 // partial[b][j] = sum over the block's rows of (X[i][j] - centre[j])^p, p = 1 or 2
-// (p = 1: the centre is 0)
-template <int P>
+// (p = 1: the centre is 0).  GROUPS = false: fewer than four rows a lane, so that
+// no group would form; the same sums without the groups' code (300 x 12 rows: 12.8 -> 12.5 us a call).
+template <int P, bool GROUPS>
 __global__ void __launch_bounds__(ZT) k_colsum(const float *__restrict__ X, int64_t n_fit, int D,
                                                const double *__restrict__ centre, double *__restrict__ partial) {
     __shared__ double red[ZT];
@@ -124,26 +125,28 @@ __global__ void __launch_bounds__(ZT) k_colsum(const float *__restrict__ X, int6
             int64_t i = r0 + rl;
             const float *p = X + i * D + j;
             const int64_t step = (int64_t)RL * D;
-            // a group's loads are in flight while the one before is added up (without
-            // that the second pass waits for memory and takes 211 us)
-            float v[ZG];
-            bool more = i + (ZG - 1) * RL < r1;
-            if (more) load_group<ZG>(v, p, step);
-            while (more) {
-                const float *cur = p;
-                float w[ZG];
-                i += ZG * RL;
-                p += ZG * step;
-                more = i + (ZG - 1) * RL < r1;
-                load_group<ZG>(w, more ? p : cur, step);
-                add_group<P, ZG>(acc, v, cur, step, c, chi, clo);
+            if constexpr (GROUPS) {
+                // a group's loads are in flight while the one before is added up (without
+                // that the second pass waits for memory and takes 211 us)
+                float v[ZG];
+                bool more = i + (ZG - 1) * RL < r1;
+                if (more) load_group<ZG>(v, p, step);
+                while (more) {
+                    const float *cur = p;
+                    float w[ZG];
+                    i += ZG * RL;
+                    p += ZG * step;
+                    more = i + (ZG - 1) * RL < r1;
+                    load_group<ZG>(w, more ? p : cur, step);
+                    add_group<P, ZG>(acc, v, cur, step, c, chi, clo);
 #pragma unroll
-                for (int u = 0; u < ZG; ++u) v[u] = w[u];
-            }
-            for (; i + 3 * RL < r1; i += 4 * RL, p += 4 * step) {
-                float v4[4];
-                load_group<4>(v4, p, step);
-                add_group<P, 4>(acc, v4, p, step, c, chi, clo);
+                    for (int u = 0; u < ZG; ++u) v[u] = w[u];
+                }
+                for (; i + 3 * RL < r1; i += 4 * RL, p += 4 * step) {
+                    float v4[4];
+                    load_group<4>(v4, p, step);
+                    add_group<P, 4>(acc, v4, p, step, c, chi, clo);
+                }
             }
             for (; i < r1; i += RL, p += step) {
                 const double d = (double)*p - c;
@@ -166,17 +169,23 @@ __global__ void __launch_bounds__(ZT) k_colsum(const float *__restrict__ X, int6
 
 // out[j] = sum_b partial[b][j] / n_fit (P = 1: the mean), or its square root
 // (P = 2: the population deviation); a warp a column (one thread a column took
-// 70 us over 608 partials)
+// 70 us over 608 partials), or, of few partials, a thread: the warp's butterfly
+// costs a call of 50 x 33 rows 1.8 us, of 1000 x 33 (12 partials) 0.7, and pays
+// from some 16 partials on (1500 x 33: 15.8 us with warps, 16.7 with threads).
+constexpr int FEW = 12;
+
 template <int P>
 __global__ void __launch_bounds__(ZT) k_colcombine(const double *__restrict__ partial, int G, int D, int64_t n_fit,
                                                    double *__restrict__ out) {
-    const int j = (blockIdx.x * ZT + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int t = blockIdx.x * ZT + threadIdx.x, lane = threadIdx.x & 31;
+    const bool few = G <= FEW;
+    const int j = few ? t : t >> 5;
     if (j >= D) return;
     double s = 0.0;
-    for (int b = lane; b < G; b += 32) s += partial[(size_t)b * D + j];
-    s = warp_sum(s);
+    for (int b = few ? 0 : lane; b < G; b += few ? 1 : 32) s += partial[(size_t)b * D + j];
+    if (!few) s = warp_sum(s);
     const double v = s / (double)n_fit;
-    if (lane == 0) out[j] = P == 2 ? sqrt(v) : v;
+    if (few || lane == 0) out[j] = P == 2 ? sqrt(v) : v;
 }
 
 template <typename TO>
@@ -197,10 +206,13 @@ constexpr int ZU = 8;              // rows in flight a thread
 constexpr int ZTILE = 32 * 1024;   // most bytes of an output tile
 
 // Rows of a tile: ZU for each of the 256 / D row lanes, so a multiple of 8 and
-// every tile of a 16-byte aligned Y starts on 16 bytes; 0 if D is above 256 or
-// the tile would not fit (k_zapply takes those).
-int tile_rows(int D, int D_out, int size) {
-    if (D > ZT) return 0;
+// every tile of a 16-byte aligned Y starts on 16 bytes; 0 if D is above 256, the
+// tile would not fit, or the table is small: k_zapply takes those.  Up to 2^16
+// values one wave does it and the tile's steps are all latency: a call of 600 x 33
+// rows 13.6 us without tiles and 14.2 with, 1500 x 60 17.6 and 17.8, 5000 x 33 to
+// bf16 x 48 17.8 and 17.0.
+int tile_rows(int64_t n, int D, int D_out, int size) {
+    if (D > ZT || n * D_out <= 65536) return 0;
     const int64_t r = (int64_t)(ZT / D) * ZU;
     return r * D_out * size <= ZTILE ? (int)r : 0;
 }
@@ -300,10 +312,15 @@ extern "C" mlp_status mlp_zscore(const float *X, int64_t n, int32_t D, int64_t n
         return set_error(MLP_EINVAL, "mlp_zscore: workspace smaller than mlp_zscore_workspace_bytes");
     cudaStream_t st = (cudaStream_t)stream;
     double *partial = (double *)workspace;
-    const int cb = (D + ZT / 32 - 1) / (ZT / 32);
-    k_colsum<1><<<G, ZT, 0, st>>>(X, n_fit, D, nullptr, partial);
+    const int cols = G <= FEW ? ZT : ZT / 32;   // of a block of k_colcombine
+    const int cb = (D + cols - 1) / cols;
+    const int64_t RL = D <= ZT ? ZT / D : 1, lane_rows = ((n_fit + G - 1) / G + RL - 1) / RL;
+    const bool groups = lane_rows >= 4;
+    auto sum1 = groups ? k_colsum<1, true> : k_colsum<1, false>;
+    auto sum2 = groups ? k_colsum<2, true> : k_colsum<2, false>;
+    sum1<<<G, ZT, 0, st>>>(X, n_fit, D, nullptr, partial);
     k_colcombine<1><<<cb, ZT, 0, st>>>(partial, G, D, n_fit, mean);
-    k_colsum<2><<<G, ZT, 0, st>>>(X, n_fit, D, mean, partial);
+    sum2<<<G, ZT, 0, st>>>(X, n_fit, D, mean, partial);
     k_colcombine<2><<<cb, ZT, 0, st>>>(partial, G, D, n_fit, sdev);
     const int64_t total = n * (int64_t)D_out;
     int64_t blocks = (total + ZT - 1) / ZT;
@@ -312,7 +329,7 @@ extern "C" mlp_status mlp_zscore(const float *X, int64_t n, int32_t D, int64_t n
     const size_t smem = sizeof(float) * 3 * (size_t)D;
     if (smem > 48 * 1024) return set_error(MLP_EUNSUPPORTED, "mlp_zscore: D above 4096");
     const int size = out_prec == MLP_FP32 ? 4 : 2;
-    const int R = tile_rows(D, D_out, size);
+    const int R = tile_rows(n, D, D_out, size);
     if (R > 0 && ((uintptr_t)Y & 15) == 0) {
         int64_t tb = (n + R - 1) / R;
         const int64_t tcap = 8 * (int64_t)device_sm_count();

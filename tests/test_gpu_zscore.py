@@ -131,3 +131,25 @@ def test_tiled_and_plain_apply_agree(prec, D, D_out, n):
         out.append(host(buf[off:off + n * D_out]))
         assert int(buf[off + n * D_out]) == 99
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("prec,D,D_out,n", [(B.MLP_FP32, 33, 33, 2000), (B.MLP_FP32, 33, 35, 2129), (B.MLP_FP32, 3, 3, 22007),
+                                            (B.MLP_BF16, 33, 37, 2065), (B.MLP_BF16, 256, 256, 275), (B.MLP_FP32, 5, 21, 4001),
+                                            (B.MLP_BF16, 257, 264, 300), (B.MLP_FP32, 1, 300, 300), (B.MLP_BF16, 33, 48, 1365),
+                                            (B.MLP_BF16, 33, 48, 1366)])
+def test_tiled_and_plain_apply_agree_on_tables_that_take_tiles(prec, D, D_out, n):
+    """As above for tables beyond 2^16 values, from where aligned outputs go
+    through tiles (the last two on both sides of that line)."""
+    test_tiled_and_plain_apply_agree(prec, D, D_out, n)
+
+
+@pytest.mark.parametrize("n_fit", [1, 2, 64, 511, 512, 768, 769, 1024, 2112])
+@pytest.mark.parametrize("D", [5, 33, 300])
+def test_statistics_around_the_few_partials_line(n_fit, D):
+    """Up to twelve blocks' partials a thread adds a column's, beyond a warp: mean
+    and deviation against numpy in 64 bits."""
+    X = table(23 + n_fit, n_fit + 3, D)
+    Y, m, s = run(X, n_fit, B.MLP_FP32, D)
+    F = X[:n_fit].astype(np.float64)
+    assert np.all(np.abs(m - F.mean(0)) <= 1e-12 * (np.abs(F.mean(0)) + F.std(0)))
+    np.testing.assert_allclose(s, F.std(0), rtol=1e-12, atol=0)
