@@ -159,7 +159,10 @@ __global__ void __launch_bounds__(NTH) k_fwd_hidden(int D, int H, int64_t n, int
             T zp = T(0), h[4];
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
-                h[jj] = Act<ACT>::f(acc[i][jj] + bj[jj]);
+                // (FP64: an activation costs as much as 50 multiply-adds, so a last tile of one
+                // to three units skips what no thread needs: 16-385, 8000 rows 277 -> 253 us)
+                if (sizeof(T) == 8 && j0 + jj >= H) h[jj] = T(0);
+                else h[jj] = Act<ACT>::f(acc[i][jj] + bj[jj]);
                 if (j0 + tx * 4 + jj < H) zp = fma(h[jj], wj[jj], zp);
             }
             if (hid && row < n) {
@@ -578,8 +581,9 @@ void launch_hidden(int D, int H, int64_t n, const void *X, const void *W1, const
         cudaFuncSetAttribute((void *)k_fwd_hidden<T, TX, ACT, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int64_t gx = cdiv(n, 16 * RPT);
     const int ntj = (int)cdiv(H, TJ);
-    // unit tiles a block: few enough that the grid has eight blocks an SM
-    int64_t gy = cdiv(8 * (int64_t)sms, gx);
+    // unit tiles a block: few enough that the grid has eight blocks an SM, or in
+    // FP64, where a block of several tiles takes long, 32 (64-512, 17394 rows: 1403 and 1356 us)
+    int64_t gy = cdiv((sizeof(T) == 8 ? 32 : 8) * (int64_t)sms, gx);
     if (gy > ntj) gy = ntj;
     const int tpb = (int)cdiv(ntj, gy);
     k_fwd_hidden<T, TX, ACT, RPT><<<dim3((unsigned)gx, (unsigned)cdiv(ntj, tpb)), NTH, smem, st>>>(

@@ -222,3 +222,22 @@ def test_scores_in_pieces_agree_with_scores_at_once(prec, D, H):
     o = host(whole).astype(np.float64)
     assert np.array_equal(host(lab), (o >= 0.5).astype(np.int8))
     assert np.all(np.abs(o - 0.5)[host(lab) != host(labp)] <= FWD_TOL)
+
+
+@pytest.mark.parametrize("n,D,H", [(1, 16, 65), (777, 16, 66), (4096, 5, 67), (2500, 16, 385), (9000, 70, 130)])
+@pytest.mark.parametrize("act", [0, 1])
+def test_fp64_forward_with_a_last_tile_of_few_units(n, D, H, act):
+    """One, two and three units in the last tile of 64 (activations that no thread
+    needs are skipped there), with and without stored activations."""
+    import torch
+    X, _, W = problem(7800 + n, n, D, H)
+    t = [dev(np.asarray(a, np.float64)) for a in (X, *W)]
+    nb = B.mlp_workspace_bytes(B.MLP_FP64, D, H, n)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    h_ref, o_ref = oracle.forward(X, Params(*[np.asarray(a, np.float64) for a in W]), act)
+    for store in (False, True):
+        hd, o = torch.zeros((n, H), device="cuda", dtype=torch.float64), torch.zeros(n, device="cuda", dtype=torch.float64)
+        B.mlp_forward_w(B.MLP_FP64, act, D, H, n, *t, hd if store else None, o, ws, nb, stream())
+        assert rel_err_elem(host(o), o_ref) <= 1e-12
+        if store:
+            assert rel_err_norm(host(hd), h_ref) <= 1e-12
