@@ -100,6 +100,40 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// grid_barrier with its wait out of line.  Inlined, the wait changes which
+// registers the sigmoid's tile loop spills: 16-512, 678124 rows in one step 236 ->
+// 250 us, 40-1536, 883136 rows 918 -> 932; so 239 and 917.  The tanh kernel's loop
+// is the faster with the wait inlined (48-2048, mini-batches of 8192: 1045 us an
+// epoch of 2^18 rows, 1077 out of line).
+__device__ __noinline__ int slice_wait(unsigned long long *bar, unsigned long long target, int *status) {
+    const unsigned long long t0 = global_ns();
+    for (int it = 1; ld_acquire(bar) < target; ++it) {
+        if ((it & 15) != 0) continue;
+        if (ld_volatile(status) & ST_TIMEOUT) return 0;
+        if (global_ns() - t0 > WAIT_LIMIT_NS) {
+            atomicOr(status, ST_TIMEOUT);
+            return 0;
+        }
+        if (it > 256) __nanosleep(64);
+    }
+    return 1;
+}
+template <int ACT>
+__device__ __forceinline__ bool slice_barrier(unsigned long long *bar, unsigned long long target, int *status) {
+    if constexpr (ACT == MLP_ACT_TANH) {
+        return grid_barrier(bar, target, status);
+    } else {
+        __shared__ int s_ok;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(bar), "l"(1ull) : "memory");
+            s_ok = slice_wait(bar, target, status);
+        }
+        __syncthreads();
+        return s_ok != 0;
+    }
+}
+
 template <int ACT>
 __global__ void __launch_bounds__(NT, 1) k_tc_cluster(const __grid_constant__ CUtensorMap tmap, ClArgs a) {
     // Launch-shape check before any tensor-memory, cluster or peer access: the
@@ -460,7 +494,7 @@ __global__ void __launch_bounds__(NT, 1) k_tc_cluster(const __grid_constant__ CU
             if (!ok) break;
             unsigned long long *sbar = a.bar + 16 * crank;
             target += (unsigned long long)K;
-            if (!grid_barrier(sbar, target, a.status)) {
+            if (!slice_barrier<ACT>(sbar, target, a.status)) {
                 ok = false;
                 break;
             }
@@ -510,7 +544,7 @@ __global__ void __launch_bounds__(NT, 1) k_tc_cluster(const __grid_constant__ CU
                 if (bad) atomicOr(a.status, ST_NONFINITE);
             }
             target += (unsigned long long)K;
-            if (!grid_barrier(sbar, target, a.status)) {
+            if (!slice_barrier<ACT>(sbar, target, a.status)) {
                 ok = false;
                 break;
             }
