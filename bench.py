@@ -523,7 +523,7 @@ def run_c0(args, rank, world, local):
         "accuracy": acc,
         "plain_fp32": {"value": units * len(t_plain) / T_p, "unit": "sample-steps/s",
                        "ms_per_step": T_p / len(t_plain) * 1e3,
-                       "path": "mlp_step_plain, one call (five kernels) per epoch",
+                       "path": "mlp_step_plain, one call (four kernels) per epoch",
                        "speedup_of_fused": (units * args.steps / T_f) / (units * len(t_plain) / T_p)},
         "e2e": {"value": units * len(t_e2e) / T_e, "unit": "sample-steps/s",
                 "h2d_bytes_per_step": C0_TRAIN * D_IN * 4 + C0_TRAIN * 4, "d2h_bytes_per_step": 8 * C0_EPOCHS,

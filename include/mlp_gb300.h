@@ -138,9 +138,9 @@ mlp_status mlp_grad_sum(const float *parts, const double *loss_parts,
                         double loss_scale, float *out, double *loss_acc,
                         void *stream);
 
-/* One training step by the plain path: separate forward, output, gradient,
- * reduction and update kernels with the hidden activations materialised in
- * device memory.  Same result as one full-batch epoch of mlp_train_epochs. */
+/* One training step by the plain path: separate forward, output and gradient
+ * kernels and one for reduction, update and loss, with the hidden activations
+ * materialised in device memory.  Same result as one full-batch epoch of mlp_train_epochs. */
 mlp_status mlp_step_plain(mlp_t net, const void *X, const void *y, int64_t n,
                           double *loss, void *stream);
 
@@ -304,7 +304,8 @@ mlp_status mlp_batch_check(mlp_batch_t b, void *stream);
  * the shapes a plan allows and keeps the fastest).  Every shape runs the same
  * method and meets the same FP32 bars against the oracle; a given shape is
  * bitwise reproducible, two shapes differ by the order of their FP32 sums.
- *   0  one hidden unit a lane, blocks of 8 warps, two per SM (any D <= 64);
+ *   0  one hidden unit a lane, blocks of 8 warps, two per SM, or one in plans
+ *      of at most one net an SM, with the same bits (any D <= 64);
  *   1  two hidden units a lane (each row word read from shared memory feeds
  *      two multiply-adds), blocks of 4 warps, two per SM, one row in flight
  *      per lane (D <= 36);
