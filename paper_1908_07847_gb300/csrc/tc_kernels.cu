@@ -37,6 +37,10 @@
 // runtime loop).  1024 nets 48-256-1 of 4096 to 16384 rows, 8 epochs: 13.95 ms
 // before, 12.12 ms now; issue slots bind next (61 % busy, 14,200 warp
 // instructions a tile).
+// For H = 128 a group has one unit block, so the serial part of a half tile shows:
+// with 40 to 56 inputs within 5 % of the form before either way, with 8 to 32 up
+// to 14 % slower (27 nets of 500 to 2100 rows, D = 16: 273 and 297 us).  That form
+// is not kept for such nets: a net's bits would follow what else is in its plan.
 //
 // Roles: warp 0 sets the ones column and issues the forward MMAs, warp 1 the TMA
 // loads and the gradient MMAs, warps 2..17 run the epilogue.  Every wait is

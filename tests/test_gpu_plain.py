@@ -241,3 +241,25 @@ def test_fp64_forward_with_a_last_tile_of_few_units(n, D, H, act):
         assert rel_err_elem(host(o), o_ref) <= 1e-12
         if store:
             assert rel_err_norm(host(hd), h_ref) <= 1e-12
+
+
+@pytest.mark.parametrize("D,H,n", [(40, 2000, 9000), (33, 516, 20011), (64, 388, 8300)])
+def test_stored_activations_of_plain_tiles(D, H, n):
+    """Activations and outputs of tiles outside the parts' range (tiny and huge
+    values in some rows, a tiny weight in the last block of units) beside tiles
+    within it, with remainders of rows and units: the bound of an FP32 sum of
+    D + 1 terms and 1e-6 of their value for the activation."""
+    import torch
+    X, _, W = problem(7900 + D, n, D, H)
+    for r, v in zip(range(9, n, 300), [1e-33, -3e-32, 2.0 ** 61, -1e-36] * n):
+        X[r, r % D] = v
+    W[0][H - 2, 1] = -1e-33
+    t = [dev(np.asarray(a, np.float32)) for a in (X, *W)]
+    hd, o = torch.zeros((n, H), device="cuda"), torch.zeros(n, device="cuda")
+    nb = B.mlp_workspace_bytes(B.MLP_FP32, D, H, n)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    B.mlp_forward_w(B.MLP_FP32, B.MLP_ACT_SIGMOID, D, H, n, *t, hd, o, ws, nb, stream())
+    h_ref, o_ref = oracle.forward(X, Params(*W))
+    assert rel_err_elem(host(o), o_ref) <= FWD_TOL
+    size = np.abs(X.astype(np.float64)) @ np.abs(W[0].astype(np.float64)).T + np.abs(W[1])
+    assert np.all(np.abs(host(hd) - h_ref) <= (D + 1) * 2.0 ** -24 * size + 1e-6 * np.abs(h_ref))
